@@ -12,6 +12,7 @@
 #include <type_traits>
 
 #include "kbc_collide.cuh"
+#include "kbc_ff.cuh"
 
 namespace kbc {
 
@@ -358,23 +359,157 @@ step_fixup(const typename C::S* __restrict__ src, typename C::S* __restrict__ ds
 
 // ---------------------------------------------------------------- init / io
 
-// f = f^eq(rho, u) (Eq. Eq) stored as deviations from W_i; computed in double.
+// f = f^eq(rho, u) (Eq. Eq) of one node, stored as deviations from W_i;
+// computed in double, in the moment form
+//   f^eq_i - W_i = W_i (q + 3 v_i.j + rho (4.5 (v_i.u)^2 - 1.5 u^2)),
+// q = rho - 1, j = rho u: 28 FP64 instructions where nine polynomials took 61.
 template <class C>
-__global__ void init_feq(const double* __restrict__ rho, const double* __restrict__ ux,
-                         const double* __restrict__ uy, typename C::S* __restrict__ dst,
-                         StepArgs a)
+__device__ __forceinline__ void feq_node(double r, double x, double y, typename C::S* __restrict__ dst,
+                                         long long n, const StepArgs& a)
 {
-    const long long total = (long long)a.nx * a.ny;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total;
-         n += (long long)gridDim.x * blockDim.x) {
-        const double r = rho[n], x = ux[n], y = uy[n];
-        const double usq15 = 1.5 * (x * x + y * y);
+    const double q = r - 1.0, jx = r * x, jy = r * y;
+    const double A = jx * x, B = jy * y, xy = 0.25 * (jx * y);
+    const double S = A + B, q9 = (1.0 / 9.0) * q;
+    const double ex = fma(1.0 / 3.0, A, fma(-1.0 / 6.0, B, q9));
+    const double ey = fma(1.0 / 3.0, B, fma(-1.0 / 6.0, A, q9));
+    const double g = fma(1.0 / 12.0, S, 0.25 * q9);
+    const double dp = g + xy, dm = g - xy, sp = jx + jy, sm = jx - jy;
+    double d[9];
+    d[4] = fma(-2.0 / 3.0, S, 4.0 * q9);
+    d[5] = fma(1.0 / 3.0, jx, ex);
+    d[3] = fma(-1.0 / 3.0, jx, ex);
+    d[7] = fma(1.0 / 3.0, jy, ey);
+    d[1] = fma(-1.0 / 3.0, jy, ey);
+    d[8] = fma(1.0 / 12.0, sp, dp);
+    d[0] = fma(-1.0 / 12.0, sp, dp);
+    d[2] = fma(1.0 / 12.0, sm, dm);
+    d[6] = fma(-1.0 / 12.0, sm, dm);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = C::from_f64(d[i], i, a.cs);
+}
+
+// out of line: the rarely taken branch of feq_pair, which keeps the order
+// of operations that the stored float and half values have always had
+template <class C>
+__device__ __noinline__ void feq_node_general(double r, double x, double y,
+                                              typename C::S* __restrict__ dst, long long n, const StepArgs& a)
+{
+    const double usq15 = 1.5 * (x * x + y * y);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const double xi = va(i) * x + vb(i) * y;
+        const double P = xi * (3.0 + 4.5 * xi) - usq15;
+        const double dev = wgt(i) * ((r - 1.0) + r * P);
+        dst[(long long)i * a.plane + n] = C::from_f64(dev, i, a.cs);
+    }
+}
+
+// Two nodes n0, n1 (n1 < 0: none) of the equilibrium for float or half
+// storage in pairs of floats, packed over the nodes: the moment form of
+// feq_node with the factors 1/9, 1/3 and 1 (float) or S, 3 S and 9 S (half
+// codes are (f - W) S / W) on q, the first- and second-order terms.  Error
+// bound: every term is a product of at most four pairs (4 2^-45) of inputs
+// with 2^-48, then at most four additions (2^-46 of M each), so 2^-42 M
+// covers it, M the sum of the terms' magnitudes (for the rest population
+// its own two terms'); the double computation's own error is 2^-50 M.
+template <class C>
+__device__ __forceinline__ void feq_pair(const double (&r)[2], const double (&x)[2], const double (&y)[2],
+                                         typename C::S* __restrict__ dst, long long n0, long long n1,
+                                         const StepArgs& a)
+{
+    using L = Lf2;
+    constexpr bool half = std::is_same<C, CodecF16>::value;
+    float h[3][2], l[3][2];
+    bool ok[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        ok[k] = split_double(r[k] - 1.0, h[0][k], l[0][k]);
+        ok[k] = split_double(x[k], h[1][k], l[1][k]) && ok[k];
+        ok[k] = split_double(y[k], h[2][k], l[2][k]) && ok[k];
+    }
+    const FF<L> q(L(h[0][0], h[0][1]), L(l[0][0], l[0][1]));
+    const FF<L> u(L(h[1][0], h[1][1]), L(l[1][0], l[1][1]));
+    const FF<L> v(L(h[2][0], h[2][1]), L(l[2][0], l[2][1]));
+    FF<L> rho = two_sum(L(1.0f), q.h);
+    rho = fast_two_sum(rho.h, rho.l + q.l);
+    const FF<L> jx = rho * u, jy = rho * v;
+    FF<L> c1, c3;
+    FF<L> q1, C9;
+    const FF<L> xy = jx * v;
+    if constexpr (half) {
+        const float S = a.cs.scale;
+        const float s3 = 3.0f * S, s9 = 9.0f * S;
+        c3 = FF<L>(L(s3), L(__fmaf_rn(3.0f, S, -s3)));
+        q1 = FF<L>(q.h, q.l) * FF<L>(L(S), L(0.0f));
+        C9 = xy * FF<L>(L(s9), L(__fmaf_rn(9.0f, S, -s9)));
+    } else {
+        c1 = FF<L>(L(ff_hi(1.0 / 9.0)), L(ff_lo(1.0 / 9.0)));
+        c3 = FF<L>(L(ff_hi(1.0 / 3.0)), L(ff_lo(1.0 / 3.0)));
+        q1 = q * c1;
+        C9 = xy;
+    }
+    const FF<L> A = (jx * u) * c3, B = (jy * v) * c3, px = jx * c3, py = jy * c3;
+    const FF<L> S3 = A + B;
+    const FF<L> ex = (q1 + A) + scale(B, -0.5f), ey = (q1 + B) + scale(A, -0.5f);
+    const FF<L> g = q1 + S3;
+    const FF<L> dp = g + C9, dm = g - C9, sp = px + py, sm = px - py;
+    FF<L> d[9];
+    d[4] = add_raw(q1, scale(S3, -0.5f));
+    d[5] = add_raw(ex, px);
+    d[3] = add_raw(ex, -px);
+    d[7] = add_raw(ey, py);
+    d[1] = add_raw(ey, -py);
+    d[8] = add_raw(dp, sp);
+    d[0] = add_raw(dp, -sp);
+    d[2] = add_raw(dm, sm);
+    d[6] = add_raw(dm, -sm);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float m4 = fabsf(q1.h.get(k)) + fabsf(A.h.get(k)) + fabsf(B.h.get(k));
+        const float m = 2.0f * m4 + fabsf(C9.h.get(k)) + fabsf(px.h.get(k)) + fabsf(py.h.get(k));
+        // below 2^-28 the inputs' cut at 2^-74 would count; above, overflow
+        bool fine = ok[k] && m > (half ? 0x1p-28f * a.cs.scale : 0x1p-28f) && m < 0x1p60f;
+        const long long n = k ? n1 : n0;
+        typename C::S out[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            const double xi = va(i) * x + vb(i) * y;
-            const double P = xi * (3.0 + 4.5 * xi) - usq15;
-            const double dev = wgt(i) * ((r - 1.0) + r * P);
-            dst[(long long)i * a.plane + n] = C::from_f64(dev, i, a.cs);
+            // the stored value is the sum over 4 (float, diagonals) or times 4 (float, rest)
+            const float w = half ? 1.0f : (wclass(i) == 0 ? 0.25f : wclass(i) == 2 ? 4.0f : 1.0f);
+            const float err = (i == 4 ? m4 : m) * (0x1p-42f * w);
+            round_sure(d[i].h.get(k) * w, d[i].l.get(k) * w, err, out[i], fine);
+        }
+        if (n >= 0) {
+            if (fine) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = out[i];
+            } else {
+                feq_node_general<C>(r[k], x[k], y[k], dst, n, a);
+            }
+        }
+    }
+}
+
+// Two nodes per thread for float and half storage (grid stride apart, so
+// that every access stays coalesced): about 200 instructions a node, two of
+// them FP64, against 67 FP64 instructions before; 4096^2 from device fields
+// 1906 -> 360 us (float), 2187 -> 372 us (half), 1635 -> 994 us (double), 80 us
+// of each the caller's copy of u into one array.
+template <class C>
+__global__ void __launch_bounds__(256)
+init_feq(const double* __restrict__ rho, const double* __restrict__ ux,
+         const double* __restrict__ uy, typename C::S* __restrict__ dst, StepArgs a)
+{
+    const long long total = (long long)a.nx * a.ny;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    if constexpr (std::is_same<C, CodecF64>::value) {
+        for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total; n += stride)
+            feq_node<C>(rho[n], ux[n], uy[n], dst, n, a);
+    } else {
+        for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total; n += 2 * stride) {
+            const long long n1 = n + stride < total ? n + stride : -1;
+            const long long m = n1 >= 0 ? n1 : n;
+            const double r[2] = {rho[n], rho[m]}, x[2] = {ux[n], ux[m]}, y[2] = {uy[n], uy[m]};
+            feq_pair<C>(r, x, y, dst, n, n1, a);
         }
     }
 }
@@ -464,26 +599,46 @@ __global__ void probe_nodes(const typename C::S* __restrict__ src, const long lo
     }
 }
 
-// rho and u of every node in double (from the stored deviations)
+// rho and u of a node in double (from the stored deviations).  Float and
+// half storage: exact integer sums, rounded once (FixedSums), so that six
+// FP64 instructions and three conversions remain of about forty; a node
+// whose values do not share a unit takes the double sums.  Bound by the FP64
+// pipe; 4096^2 moments 1106 -> 327 us (float), 1266 -> 364 us (half),
+// 828 -> 700 us (double, shared differences and rcp_pos), against 150, 127
+// and 241 us for the bytes.
 template <class C>
 __device__ __forceinline__ void node_macro(const typename C::S* __restrict__ src, long long n,
                                            const StepArgs& a, double& rho, double& ux, double& uy)
 {
+    typename C::S c[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) c[i] = src[(long long)i * a.plane + n];
+    if constexpr (fixed_of<C>::kHas) {
+        FixedSums s;
+        if (fixed_of<C>::sums(c, a.cs, s)) {
+            rho = __fma_rn(s.unit, (double)s.drho, 1.0);
+            const double ir = rcp_pos(rho) * s.unit;
+            ux = (double)s.jx * ir;
+            uy = (double)s.jy * ir;
+            return;
+        }
+    }
     double d[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) d[i] = C::to_f64(src[(long long)i * a.plane + n], i, a.cs);
-    const double drho = ((d[0] + d[8]) + (d[2] + d[6])) + ((d[1] + d[7]) + (d[3] + d[5])) + d[4];
-    const double jx = ((d[2] - d[0]) + (d[8] - d[6])) + (d[5] - d[3]);
-    const double jy = ((d[6] - d[0]) + (d[8] - d[2])) + (d[7] - d[1]);
-    rho = 1.0 + drho;
-    const double irho = 1.0 / rho;  // one division for both components
-    ux = jx * irho;
-    uy = jy * irho;
+    for (int i = 0; i < 9; ++i) d[i] = C::to_f64(c[i], i, a.cs);
+    // differences of opposite populations: j keeps its relative accuracy
+    // where it is far smaller than the populations
+    const double a08 = d[8] - d[0], a26 = d[2] - d[6];
+    rho = 1.0 + (((d[0] + d[8]) + (d[2] + d[6])) + ((d[1] + d[7]) + (d[3] + d[5])) + d[4]);
+    const double irho = rcp_pos(rho);  // one reciprocal for both components
+    ux = ((a08 + a26) + (d[5] - d[3])) * irho;
+    uy = ((a08 - a26) + (d[7] - d[1])) * irho;
 }
 
 template <class C>
-__global__ void moments(const typename C::S* __restrict__ src, double* __restrict__ rho,
-                        double* __restrict__ ux, double* __restrict__ uy, StepArgs a)
+__global__ void __launch_bounds__(256)
+moments(const typename C::S* __restrict__ src, double* __restrict__ rho,
+        double* __restrict__ ux, double* __restrict__ uy, StepArgs a)
 {
     const long long total = (long long)a.nx * a.ny;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total;
