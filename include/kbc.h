@@ -176,11 +176,12 @@ int kbc_set_gamma_mode(kbc_handle h, int mode, double gamma_fixed);
 
 /* Kernel used by kbc_step (all of them share the collision arithmetic, so
  * they give identical bits):
- *   KBC_KERNEL_AUTO  (default) the fastest choice measured on GB300 at 4096^2
- *                    and 16384^2: for F16 storage with a KBC variant the
- *                    bulk-copy kernel below where nx is a multiple of 512,
- *                    otherwise the vector-row kernel where nx is a multiple
- *                    of its row width, else the per-node kernel;
+ *   KBC_KERNEL_AUTO  (default) the fastest choice measured on GB300: the
+ *                    per-node kernel for F64, for KBC variants on small grids
+ *                    and for widths the others do not take; the bulk-copy
+ *                    kernel below for F16 storage with a KBC variant on large
+ *                    grids with nx a multiple of 512; otherwise the vector-row
+ *                    kernel where nx is a multiple of its row width;
  *   KBC_KERNEL_ROWS  the vector-row kernel where nx allows it, else the
  *                    per-node kernel;
  *   KBC_KERNEL_NODES the per-node kernel;

@@ -304,13 +304,24 @@ static int step_into(kbc_handle h, const void* src, void* dst, cudaStream_t stre
 {
     Launch L;
     L.variant = h->variant;
-    L.rows = h->kernel != KBC_KERNEL_NODES && (h->nx % (32 * vec_width(h->dtype))) == 0;
-    // AUTO takes the bulk-copy kernel for FP16 KBC (measured 1-3% faster than
-    // the vector rows there; the rows win for LBGK and for FP32 by 12-16%)
-    const bool bulk = h->kernel == KBC_KERNEL_BULK ||
-                      (h->kernel == KBC_KERNEL_AUTO && h->dtype == KBC_F16_DEV &&
-                       h->variant != KBC_LBGK);
-    L.tma = bulk && h->dtype != KBC_F64 && (h->nx % kTmaTile) == 0;
+    // AUTO takes, measured in us a step with the others in brackets:
+    // - per node for doubles (64^2 B 8.1 [rows 14.5], 2048^2 1525 [1541]), for
+    //   KBC on grids whose nodes are all resident at once (256^2 F32 B 3.1
+    //   [rows 3.4]; F16 B 2.1 [rows 2.25]) and for the widths that the other
+    //   two do not take;
+    // - bulk copies for FP16 KBC with several tiles for every resident block
+    //   (4096^2 B 136 [rows 155], 1024^2 10.3 [10.5]; 512^2 4.3 [rows 3.9]);
+    // - vector rows otherwise (4096^2 F32 B 180 [bulk 221], LBGK 172 [196]).
+    const long long total = (long long)h->nx * h->ny;
+    const bool tiles = h->dtype != KBC_F64 && h->nx % kTmaTile == 0, kbc = h->variant != KBC_LBGK;
+    const bool autok = h->kernel == KBC_KERNEL_AUTO || (h->kernel == KBC_KERNEL_BULK && !tiles);
+    const bool bulk = autok ? h->dtype == KBC_F16_DEV && kbc && total >= (long long)h->num_sms * 4096
+                            : h->kernel == KBC_KERNEL_BULK;
+    const bool rows = autok ? h->dtype != KBC_F64 && !(kbc && flat_small(h->nx, h->ny, h->num_sms))
+                            : h->kernel == KBC_KERNEL_ROWS;
+    if (bulk && tiles) L.kind = StepKind::bulk;
+    else if (rows && h->nx % (32 * vec_width(h->dtype)) == 0) L.kind = StepKind::rows;
+    else L.kind = StepKind::nodes;
     L.all_f64 = h->gamma_mode == KBC_GAMMA_EXACT && h->variant != KBC_LBGK;
     L.stream = use_stream ? stream : h->stream;
     L.num_sms = h->num_sms;

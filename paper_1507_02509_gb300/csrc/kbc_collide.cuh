@@ -220,7 +220,7 @@ __device__ __forceinline__ L collide(L (&d)[9], const CollideParams<typename L::
     // a power of two, exact either way)
     L nusq15;
     if constexpr (U) nusq15 = L(-1.5) * fmaL(ux, ux, uyy);
-    else nusq15 = L(-1.5) * (uxx + uyy);
+    else nusq15 = L(-1.5) * square_sum(ux, uy);
     const L sxy = ux + uy, dxy = ux - uy;
 
     L P[9], df[9];

@@ -39,6 +39,65 @@ __device__ __forceinline__ int pull_row(int sy, const StepArgs& a)
     return sy < 0 ? sy + a.ny : (sy >= a.ny ? sy - a.ny : sy);
 }
 
+// ---------------------------------------------------------------- launches
+//
+// The kernels of a step are launched with programmatic stream serialisation:
+// the launch of a kernel and the start of its blocks overlap the end of the
+// kernel before it, 0.2 us a kernel in a replayed graph (64^2, float: LBGK
+// 1.75 -> 1.55 us a step, B with its guard pass 3.02 -> 2.70 us).  Every
+// kernel starts with chain_enter(), which waits until the one before has
+// completed and its writes are visible; nothing is read or written before
+// that, and every thread passes it, so a kernel's completion still implies
+// that of all before it.  No kernel lets the next one start early
+// (griddepcontrol.launch_dependents): blocks placed while others still run
+// crowd onto the SMs that empty first (200^2 double LBGK 8.9 -> 15.6 us a
+// step, 512^2 float B 5.1 -> 6.5 us).
+__device__ __forceinline__ void chain_enter()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Loads of the field.  Coherent and ordered after chain_enter(): the kernel
+// before may still be writing the field while this kernel's blocks start, so
+// the read-only path, whose loads the compiler may move, is not for them.
+__device__ __forceinline__ unsigned short ld_field(const unsigned short* p)
+{
+    unsigned v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return (unsigned short)v;
+}
+__device__ __forceinline__ int ld_count(const int* p)
+{
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_field(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_field(const double* p)
+{
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_field(const uint2* p)
+{
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ld_field(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
 // ---------------------------------------------------------------- vectors
 
 template <int BYTES> struct RawT;
@@ -57,7 +116,7 @@ struct Vec {
     __device__ __forceinline__ static void load(const S* p, S (&v)[NV])
     {
         U u;
-        u.r = __ldg(reinterpret_cast<const Raw*>(p));
+        u.r = ld_field(reinterpret_cast<const Raw*>(p));
 #pragma unroll
         for (int k = 0; k < NV; ++k) v[k] = u.s[k];
     }
@@ -181,6 +240,7 @@ step_rows(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst
     const int y = blockIdx.x / nbx;
     const int bx = blockIdx.x - y * nbx;
     const int x0 = (bx * BLOCK + threadIdx.x) * NV;
+    chain_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.fix_count)
         a.fix_count[a.fix_slot ^ 1] = 0;  // free the other counter for the next step
     if (x0 >= a.nx) return;               // whole warps only (nx % (32 NV) == 0)
@@ -200,10 +260,10 @@ step_rows(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst
         Vec<S, NV>::load(row + x0, raw[i]);
         if (ai == 1) {
             edge[i] = S(0);
-            if (lane == 0) edge[i] = __ldg(row + xl);
+            if (lane == 0) edge[i] = ld_field(row + xl);
         } else if (ai == -1) {
             edge[i] = S(0);
-            if (lane == 31) edge[i] = __ldg(row + xr);
+            if (lane == 31) edge[i] = ld_field(row + xr);
         }
     }
     T f[NV][9];
@@ -252,37 +312,92 @@ step_rows(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst
 
 // ---------------------------------------------------------------- step, nodes
 //
-// One node per thread, any nx, ny; same arithmetic as step_rows.
-template <int VAR, class C>
-__global__ void __launch_bounds__(256)
+// Any nx, ny; same arithmetic as step_rows.  Nodes are taken in memory order
+// across the rows: a warp holds 32 K consecutive nodes, each thread K of
+// them 32 apart (collided in packed lane pairs for float and half with K > 1),
+// so every load and store is coalesced whatever the width.  A warp whose
+// nodes lie in one row, away from its ends, addresses every population as
+// one offset shared by the warp plus the thread's index; the others wrap per
+// thread.  Bound by the latency of the collision: K = 4 gives it two
+// independent pairs (4095 x 4096, float B: K = 4 193 us, K = 2 248 us, one
+// node at a time 237 us; one node per thread with a 64-bit division before,
+// 281 us); float C needs 94 registers and runs at the copy bandwidth with
+// ten blocks per SM (176 us against 189 us with eight).  A grid whose nodes
+// find a thread each at once takes K = 1 (256^2, float B: 3.5 us a step
+// against 3.8 for the vector rows).  Double is bound by the FP64 pipe and
+// takes K = 1 everywhere (64^2: 8.1 us against 14.5 with the two nodes a
+// thread of the vector rows, 2048^2 1525 against 1541 us).
+constexpr int kFlatBlock = 64;
+// Nodes per thread on a grid that fills the GPU, and resident blocks per SM
+// the kernel is compiled for.
+template <int VAR, class C> constexpr int flat_nodes()
+{
+    return std::is_same<C, CodecF64>::value ? 1 : (VAR == kLBGK ? 2 : 4);
+}
+template <int VAR, class C, int K> constexpr int flat_min_blocks()
+{
+    return std::is_same<C, CodecF64>::value ? 1 : (K < 4 ? 12 : (VAR == kC || VAR == kD) ? 10 : 8);
+}
+
+template <int VAR, class C, int K>
+__global__ void __launch_bounds__(kFlatBlock, flat_min_blocks<VAR, C, K>())
 step_nodes(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst, StepArgs a)
 {
     using S = typename C::S;
     using T = typename C::T;
+    chain_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.fix_count) a.fix_count[a.fix_slot ^ 1] = 0;
-    const long long total = (long long)a.nx * a.ny;
-    const CollideParams<T>& p = params_of<T>(a);
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(n / a.nx), x = (int)(n - (long long)y * a.nx);
-        T f[9];
+    const int total = a.nx * a.ny;
+    const int lane = threadIdx.x & 31;
+    // first node of the warp (uniform), its row and column
+    const unsigned w0 = (blockIdx.x * kFlatBlock + (threadIdx.x & ~31u)) * K;
+    if (w0 >= (unsigned)total) return;
+    const int y0 = (int)(w0 / (unsigned)a.nx), x0 = (int)w0 - y0 * a.nx;
+    const bool yin = !a.ywrap || (y0 > 0 && y0 + 1 < a.ny);
+    S raw[K][9];
+    if (yin && x0 > 0 && x0 + 32 * K < a.nx) {
+        const S* base = src + w0 + lane;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            const int ai = i % 3 - 1, bi = i / 3 - 1;
-            int sx = x - ai, sy = y - bi;
-            sx = sx < 0 ? sx + a.nx : (sx >= a.nx ? sx - a.nx : sx);
-            sy = pull_row(sy, a);
-            f[i] = C::load(__ldg(src + (long long)i * a.plane + (long long)sy * a.nx + sx), i, a.cs);
-        }
-        T rho;
-        bool hit;
-        collide_node<VAR, C::kUnits>(f, p, rho, hit);
-        if (!isfinite(rho)) *a.flag = 1;
-        if constexpr (VAR != kLBGK) {
-            if (a.fix_list) record_fix(hit, (int)n, a);
-        }
+            const S* pl = base + ((long long)i * a.plane - vb(i) * (long long)a.nx - va(i));
 #pragma unroll
-        for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = C::store(f[i], i, a.cs);
+            for (int k = 0; k < K; ++k) raw[k][i] = ld_field(pl + 32 * k);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            int n = (int)w0 + 32 * k + lane;
+            if ((unsigned)n >= (unsigned)total) n = total - 1;  // idle lanes repeat the last node
+            const int y = (int)((unsigned)n / (unsigned)a.nx), x = n - y * a.nx;
+            const int ym = pull_row(y - 1, a), yp = pull_row(y + 1, a);
+            const int xl = x == 0 ? a.nx - 1 : x - 1, xr = x + 1 == a.nx ? 0 : x + 1;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const int sy = vb(i) == 1 ? ym : (vb(i) == -1 ? yp : y);
+                const int sx = va(i) == 1 ? xl : (va(i) == -1 ? xr : x);
+                raw[k][i] = ld_field(src + (long long)i * a.plane + (long long)sy * a.nx + sx);
+            }
+        }
+    }
+    T f[K][9];
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[k][i] = C::load(raw[k][i], i, a.cs);
+    bool bad = false;
+    const unsigned hits = collide_vec<VAR, C::kUnits, (K > 1)>(f, params_of<T>(a), bad);
+    if (bad) *a.flag = 1;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int n = (int)w0 + 32 * k + lane;
+        const bool live = (unsigned)n < (unsigned)total;
+        if constexpr (VAR != kLBGK) {
+            if (a.fix_list) record_fix(live && (hits >> k & 1u), n, a);
+        }
+        if (live) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = C::store(f[k][i], i, a.cs);
+        }
     }
 }
 
@@ -295,6 +410,7 @@ template <int VAR, class C>
 __global__ void __launch_bounds__(256)
 step_nodes_f64(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst, StepArgs a)
 {
+    chain_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.fix_count) a.fix_count[a.fix_slot ^ 1] = 0;
     const long long total = (long long)a.nx * a.ny;
     CollideParams<double> p = a.pd;
@@ -309,7 +425,7 @@ step_nodes_f64(const typename C::S* __restrict__ src, typename C::S* __restrict_
             int sx = x - ai, sy = y - bi;
             sx = sx < 0 ? sx + a.nx : (sx >= a.nx ? sx - a.nx : sx);
             sy = pull_row(sy, a);
-            f[i] = C::to_f64(src[(long long)i * a.plane + (long long)sy * a.nx + sx], i, a.cs);
+            f[i] = C::to_f64(ld_field(src + (long long)i * a.plane + (long long)sy * a.nx + sx), i, a.cs);
         }
         double rho;
         bool hit;
@@ -330,13 +446,14 @@ __global__ void __launch_bounds__(256)
 step_fixup(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst, StepArgs a)
 {
     using S = typename C::S;
-    const int recorded = a.fix_count[a.fix_slot];
+    chain_enter();
+    const int recorded = ld_count(a.fix_count + a.fix_slot);
     const int count = recorded < a.nx * a.ny ? recorded : a.nx * a.ny;
     if (count == 0) return;
     // node t goes to block t % gridDim.x: the few recorded nodes spread over
     // every SM's FP64 pipe instead of filling the first blocks
     for (int t = threadIdx.x * gridDim.x + blockIdx.x; t < count; t += gridDim.x * blockDim.x) {
-        const int n = a.fix_list[t];
+        const int n = ld_count(a.fix_list + t);
         const int y = n / a.nx, x = n - y * a.nx;
         double f[9];
 #pragma unroll
@@ -345,7 +462,7 @@ step_fixup(const typename C::S* __restrict__ src, typename C::S* __restrict__ ds
             int sx = x - ai, sy = y - bi;
             sx = sx < 0 ? sx + a.nx : (sx >= a.nx ? sx - a.nx : sx);
             sy = pull_row(sy, a);
-            f[i] = C::to_f64(src[(long long)i * a.plane + (long long)sy * a.nx + sx], i, a.cs);
+            f[i] = C::to_f64(ld_field(src + (long long)i * a.plane + (long long)sy * a.nx + sx), i, a.cs);
         }
         CollideParams<double> q = a.pd;
         q.guard = 0.0;

@@ -113,6 +113,14 @@ __device__ __forceinline__ Lf2 select(unsigned m, Lf2 a, Lf2 b)
     return Lf2((m & 1u) ? a.v.x : b.v.x, (m & 2u) ? a.v.y : b.v.y);
 }
 
+// a^2 + b^2 with each product and the sum rounded: in the packed lane by
+// one-node operations, which are never fused (see above)
+template <class L> __device__ __forceinline__ L square_sum(L a, L b) { return a * a + b * b; }
+__device__ __forceinline__ Lf2 square_sum(Lf2 a, Lf2 b)
+{
+    return Lf2(square_sum(Lf(a.v.x), Lf(b.v.x)).v, square_sum(Lf(a.v.y), Lf(b.v.y)).v);
+}
+
 // scalar arithmetic type -> one-node lane
 template <typename T> struct LaneOf;
 template <> struct LaneOf<float> { using type = Lf; };

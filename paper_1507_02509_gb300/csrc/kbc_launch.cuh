@@ -13,13 +13,20 @@
 
 namespace kbc {
 
+// rows: vectorised row kernel (nx % (32 * kVec) == 0); nodes: any width;
+// bulk: persistent bulk-copy kernel (nx % kTmaTile == 0, F32/F16)
+enum class StepKind { rows, nodes, bulk };
+
+// Whether every node finds a thread of its own in the first wave of
+// step_nodes: 1024 threads (16 blocks of 64) are resident per SM.
+inline bool flat_small(int nx, int ny, int num_sms) { return (long long)nx * ny <= (long long)num_sms * 1024; }
+
 struct Launch {
     const void* src;
     void* dst;
     StepArgs a;
     int variant;
-    bool rows;      // vectorised row kernel (nx % (32 * kVec) == 0)
-    bool tma;       // persistent bulk-copy kernel (nx % kTmaTile == 0, F32/F16)
+    StepKind kind;
     bool all_f64;   // whole collision in double (exact-gamma mode)
     bool fixup;     // FP64 re-evaluation pass after the step
     cudaStream_t stream;
@@ -32,6 +39,24 @@ int handle_free_error(int code, const char* msg);
 
 constexpr int kRowBlock = 64;
 constexpr int kNodeBlock = 256;
+
+// Launch with programmatic stream serialisation (the kernels start with
+// chain_enter(); see there).
+template <class... P, class... Q>
+cudaError_t launch_chained(void (*kernel)(P...), long long grid, int block, size_t smem, cudaStream_t s, Q... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 inline int grid_for(long long total, int block, int num_sms, int per_sm)
 {
@@ -47,21 +72,19 @@ cudaError_t launch_step_v(const Launch& L)
     using S = typename C::S;
     const S* src = static_cast<const S*>(L.src);
     S* dst = static_cast<S*>(L.dst);
-    if (L.all_f64) {
-        const long long total = (long long)L.a.nx * L.a.ny;
-        step_nodes_f64<VAR, C><<<grid_for(total, kNodeBlock, L.num_sms, 16), kNodeBlock, 0,
-                                 L.stream>>>(src, dst, L.a);
-        return cudaGetLastError();
-    }
+    const long long total = (long long)L.a.nx * L.a.ny;
+    if (L.all_f64)
+        return launch_chained(step_nodes_f64<VAR, C>, grid_for(total, kNodeBlock, L.num_sms, 16), kNodeBlock, 0,
+                              L.stream, src, dst, L.a);
+    cudaError_t e = cudaSuccess;
     if constexpr (!std::is_same<C, CodecF64>::value) {
-        if (L.tma) {
+        if (L.kind == StepKind::bulk) {
             constexpr size_t smem = tma_smem_bytes<S, kTmaTile>();
             constexpr int threads = kTmaTile / C::kVec + 32;
             static int per_sm = 0;  // resident CTAs per SM, from the occupancy calculator
             if (per_sm == 0) {
-                cudaError_t e = cudaFuncSetAttribute(step_tma<VAR, C, kTmaTile>,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)smem);
+                e = cudaFuncSetAttribute(step_tma<VAR, C, kTmaTile>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
                 if (e != cudaSuccess) return e;
                 int n = 0;
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_tma<VAR, C, kTmaTile>,
@@ -72,29 +95,29 @@ cudaError_t launch_step_v(const Launch& L)
             const long long tiles = (long long)(L.a.nx / kTmaTile) * L.a.ny;
             long long grid = (long long)L.num_sms * per_sm;
             if (grid > tiles) grid = tiles;
-            step_tma<VAR, C, kTmaTile><<<(unsigned)grid, threads, smem, L.stream>>>(src, dst, L.a);
-            if constexpr (VAR != kLBGK) {
-                if (L.fixup)
-                    step_fixup<VAR, C><<<L.num_sms * 2, kNodeBlock, 0, L.stream>>>(src, dst, L.a);
-            }
-            return cudaGetLastError();
+            e = launch_chained(step_tma<VAR, C, kTmaTile>, grid, threads, smem, L.stream, src, dst, L.a);
         }
     }
-    if (L.rows) {
+    if (L.kind == StepKind::rows) {
         constexpr int NV = C::kVec;
         const int nbx = (L.a.nx + kRowBlock * NV - 1) / (kRowBlock * NV);
-        step_rows<VAR, C, NV, kRowBlock>
-            <<<(unsigned)((long long)nbx * L.a.ny), kRowBlock, 0, L.stream>>>(src, dst, L.a, nbx);
-    } else {
-        const long long total = (long long)L.a.nx * L.a.ny;
-        step_nodes<VAR, C><<<grid_for(total, kNodeBlock, L.num_sms, 16), kNodeBlock, 0, L.stream>>>(
-            src, dst, L.a);
+        e = launch_chained(step_rows<VAR, C, NV, kRowBlock>, (long long)nbx * L.a.ny, kRowBlock, 0, L.stream, src,
+                           dst, L.a, nbx);
+    } else if (L.kind == StepKind::nodes) {
+        constexpr int K = flat_nodes<VAR, C>();
+        if (K > 1 && !flat_small(L.a.nx, L.a.ny, L.num_sms)) {
+            constexpr int per = kFlatBlock * K;
+            e = launch_chained(step_nodes<VAR, C, K>, (total + per - 1) / per, kFlatBlock, 0, L.stream, src, dst, L.a);
+        } else {
+            e = launch_chained(step_nodes<VAR, C, 1>, (total + kFlatBlock - 1) / kFlatBlock, kFlatBlock, 0, L.stream,
+                               src, dst, L.a);
+        }
     }
     if constexpr (VAR != kLBGK) {
-        if (L.fixup)
-            step_fixup<VAR, C><<<L.num_sms * 2, kNodeBlock, 0, L.stream>>>(src, dst, L.a);
+        if (L.fixup && e == cudaSuccess)
+            e = launch_chained(step_fixup<VAR, C>, L.num_sms * 2, kNodeBlock, 0, L.stream, src, dst, L.a);
     }
-    return cudaGetLastError();
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <class C>

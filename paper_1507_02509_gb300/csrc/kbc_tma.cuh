@@ -182,7 +182,6 @@ step_tma(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst,
     const int my_tiles = first < tiles ? (tiles - 1 - first) / stride + 1 : 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.fix_count) a.fix_count[a.fix_slot ^ 1] = 0;
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < kTmaStages; ++s) {
@@ -192,6 +191,8 @@ step_tma(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst,
         fence_mbar_init();
     }
     __syncthreads();
+    chain_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0 && a.fix_count) a.fix_count[a.fix_slot ^ 1] = 0;
 
     if (warp == NCW) {
         // ---------------------------------------------------------- producer
