@@ -8,6 +8,7 @@
 
 #include "kbc_adjoint.cuh"
 #include "kbc_adjoint_async.cuh"
+#include "kbc_guard.cuh"
 #include "kbc_kernels.cuh"
 #include "kbc_tma.cuh"
 
@@ -114,8 +115,18 @@ cudaError_t launch_step_v(const Launch& L)
         }
     }
     if constexpr (VAR != kLBGK) {
-        if (L.fixup && e == cudaSuccess)
-            e = launch_chained(step_fixup<VAR, C>, L.num_sms * 2, kNodeBlock, 0, L.stream, src, dst, L.a);
+        if (L.fixup && e == cudaSuccess) {
+            if constexpr (std::is_same<C, CodecF32>::value) {
+                GuardParams gp;
+                gp.n2b_h = (float)(-L.a.pd.two_beta);
+                gp.n2b_l = (float)(-L.a.pd.two_beta - (double)gp.n2b_h);
+                gp.nb = (float)(-L.a.pd.one_m_2beta);
+                gp.settle = (double)L.a.pf.guard <= kGuardSettle;
+                e = launch_chained(step_guard<VAR>, L.num_sms, kGuardBlock, 0, L.stream, src, dst, L.a, gp);
+            } else {
+                e = launch_chained(step_fixup<VAR, C>, L.num_sms * 2, kNodeBlock, 0, L.stream, src, dst, L.a);
+            }
+        }
     }
     return e == cudaSuccess ? cudaGetLastError() : e;
 }

@@ -263,7 +263,7 @@ step_tma(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst,
         // storage units (FP16): node pairs in packed FP32x2 arithmetic
         const unsigned hits = collide_vec<VAR, C::kUnits, C::kUnits>(f, p, bad);
         if constexpr (VAR != kLBGK) {
-            if (a.fix_list) record_fix_mask<NV>(hits, y * a.nx + x0 + lx, a);
+            if (a.fix_list) record_fix<NV>(hits, y * a.nx + x0 + lx, 1, a);
         }
         const long long o = (long long)y * a.nx + x0 + lx;
 #pragma unroll
