@@ -160,6 +160,17 @@ int kbc_create_slab(int nx, int ny, int variant, double beta, int dtype, kbc_han
 int kbc_halo_send(kbc_handle h, int face, int full, void* buf);
 int kbc_halo_recv(kbc_handle h, int face, int full, const void* buf);
 
+/* nsteps steps of a grid whose y-slabs are all handles of this process on one
+ * device and stream: slabs[0 .. parts) from the lowest rows to the highest,
+ * periodic, each initialised, with the same nx and storage.  Before every
+ * step the boundary rows go straight into the neighbours' ghost rows (what
+ * kbc_halo_send and kbc_halo_recv move through a buffer), in one kernel for
+ * all slabs; the field is that of the exchange and kbc_step(slab, 1).
+ * Asynchronous like kbc_step.  Failures are described by
+ * kbc_last_error(NULL): KBC_ERR_ARG for handles that do not fit together,
+ * KBC_ERR_STATE for one that is not initialised. */
+int kbc_slabs_step(int parts, const kbc_handle* slabs, int nsteps);
+
 /* Bytes of one face's halo: 3 nx (full = 0) or 9 nx (full = 1) stored
  * elements. */
 int kbc_halo_bytes(kbc_handle h, int full, size_t* bytes);

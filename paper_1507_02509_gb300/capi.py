@@ -55,6 +55,7 @@ SIGNATURES = {
     "kbc_init_grad": (_i, [_vp, _vp, _vp]),
     "kbc_set_populations": (_i, [_vp, _vp]),
     "kbc_get_populations": (_i, [_vp, _vp]),
+    "kbc_slabs_step": (_i, [_i, ctypes.POINTER(_vp), _i]),
     "kbc_step": (_i, [_vp, _i]),
     "kbc_sync": (_i, [_vp, _d]),
     "kbc_probe": (_i, [_vp, _i, _vp, _vp]),
@@ -151,6 +152,11 @@ def kbc_halo_send(h, face: int, full: int, buf):
 
 def kbc_halo_recv(h, face: int, full: int, buf):
     return check(h, load().kbc_halo_recv(h, int(face), int(full), ptr(buf)))
+
+
+def kbc_slabs_step(handles, nsteps: int):
+    hs = (ctypes.c_void_p * len(handles))(*[h.value for h in handles])
+    return check(None, load().kbc_slabs_step(len(handles), hs, int(nsteps)))
 
 
 def kbc_halo_bytes(h, full: int = 0) -> int:

@@ -510,8 +510,8 @@ __device__ __forceinline__ double adj_node_f64(const typename C::S* __restrict__
         int sx = x - ai, sy = y - bi;
         sx = sx < 0 ? sx + a.nx : (sx >= a.nx ? sx - a.nx : sx);
         sy = sy < 0 ? sy + a.ny : (sy >= a.ny ? sy - a.ny : sy);
-        dd[i] = C::to_f64(g[(long long)i * a.plane + (long long)sy * a.nx + sx], i, a.cs);
-        ll[i] = (double)lam_in[(long long)i * a.plane + n];
+        dd[i] = C::to_f64(ld_field(g + (long long)i * a.plane + (long long)sy * a.nx + sx), i, a.cs);
+        ll[i] = (double)ld_field(lam_in + (long long)i * a.plane + n);
     }
     CollideParams<double> q = a.pd;
     q.guard = 0.0;
@@ -547,8 +547,8 @@ __device__ __forceinline__ double adj_node(const typename C::S* __restrict__ g,
         const int ai = i % 3 - 1, bi = i / 3 - 1;
         const long long off = (long long)i * a.plane + (bi == 1 ? dn : (bi == -1 ? up : 0)) +
                               (ai == 1 ? cl : (ai == -1 ? cr : 0));
-        d[i] = C::decode(g[off + t], i, a.cs);
-        lam[i] = lam_in[(long long)i * a.plane + t];
+        d[i] = C::decode(ld_field(g + off + t), i, a.cs);
+        lam[i] = ld_field(lam_in + (long long)i * a.plane + t);
     }
     T bbar;
     const bool guarded = collide_adjoint<VAR>(d, lam, p, mu, bbar);
@@ -586,6 +586,7 @@ adj_step(const typename C::S* __restrict__ g, const typename C::T* __restrict__ 
          StepArgs a)
 {
     using T = typename C::T;
+    chain_enter();
     const CollideParams<T>& p = params_of<T>(a);
     const int nbx = (a.nx + kAdjBlock - 1) / kAdjBlock;
     const int segs = nbx * a.ny;  // nx * ny < 2^31
@@ -626,12 +627,13 @@ adj_fixup(const typename C::S* __restrict__ g, const typename C::T* __restrict__
           typename C::T* __restrict__ lam_out, double* __restrict__ part, unsigned* __restrict__ fixmask,
           StepArgs a)
 {
+    chain_enter();
     const long long total = (long long)a.nx * a.ny;
     const long long words = (total + 31) >> 5;
     double bsum = 0.0;
     for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < words;
          w += (long long)gridDim.x * blockDim.x) {
-        unsigned m = fixmask[w];
+        unsigned m = (unsigned)ld_count(reinterpret_cast<const int*>(fixmask + w));
         if (m == 0u) continue;
         fixmask[w] = 0u;
         while (m) {

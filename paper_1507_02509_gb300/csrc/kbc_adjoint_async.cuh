@@ -42,6 +42,7 @@ adj_step_async(const float* __restrict__ g, const float* __restrict__ lam_in,
 {
     // [stage][operand][thread]: consecutive threads use consecutive banks
     __shared__ float slot[2][18][kAdjBlock];
+    chain_enter();
     const CollideParams<float>& p = a.pf;
     const int nbx = (a.nx + kAdjBlock - 1) / kAdjBlock;
     const int segs = nbx * a.ny;  // nx * ny < 2^31

@@ -44,13 +44,13 @@ constexpr int kNodeBlock = 256;
 // Launch with programmatic stream serialisation (the kernels start with
 // chain_enter(); see there).
 template <class... P, class... Q>
-cudaError_t launch_chained(void (*kernel)(P...), long long grid, int block, size_t smem, cudaStream_t s, Q... args)
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, Q... args)
 {
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -234,13 +234,24 @@ inline int adj_blocks(long long total, int num_sms) { return grid_for(total, 256
 // asynchronous copies (adj_step_async); the other storages load them node
 // by node (adj_step).
 template <int VAR, class C>
-void launch_adj_step_v(const typename C::S* g, const typename C::T* li, typename C::T* lo,
-                       double* part, unsigned* fixmask, int nblocks, const StepArgs& a, cudaStream_t s)
+cudaError_t launch_adj_step_v(const typename C::S* g, const typename C::T* li, typename C::T* lo,
+                              double* part, unsigned* fixmask, int nblocks, const StepArgs& a, cudaStream_t s)
 {
+    cudaError_t e;
     if constexpr (std::is_same<C, CodecF32>::value)
-        adj_step_async<VAR><<<nblocks, kAdjBlock, 0, s>>>(g, li, lo, part, fixmask, a);
+        e = launch_chained(adj_step_async<VAR>, nblocks, kAdjBlock, 0, s, g, li, lo, part, fixmask, a);
     else
-        adj_step<VAR, C><<<nblocks, kAdjBlock, 0, s>>>(g, li, lo, part, fixmask, a);
+        e = launch_chained(adj_step<VAR, C>, nblocks, kAdjBlock, 0, s, g, li, lo, part, fixmask, a);
+    if constexpr (VAR != kLBGK && !std::is_same<typename C::T, double>::value) {
+        // the double redo scans one mask word per thread: a grid sized to the
+        // mask (at most the step's), so small grids do not pay for idle blocks;
+        // its beta partial sums land in part[0 .. fblocks) in a fixed order
+        const long long words = ((long long)a.nx * a.ny + 31) / 32;
+        const int fblocks = (int)((words + 255) / 256 < nblocks ? (words + 255) / 256 : nblocks);
+        if (e == cudaSuccess)
+            e = launch_chained(adj_fixup<VAR, C>, fblocks, 256, 0, s, g, li, lo, part, fixmask, a);
+    }
+    return e;
 }
 
 template <class C>
@@ -253,27 +264,16 @@ cudaError_t launch_adj_step(int variant, const void* g, const void* lam_in, void
     const S* gp = static_cast<const S*>(g);
     const T* li = static_cast<const T*>(lam_in);
     T* lo = static_cast<T*>(lam_out);
-    constexpr bool fix = !std::is_same<T, double>::value;
-    // the double redo scans one mask word per thread: a grid sized to the
-    // mask (at most the step's), so small grids do not pay for idle blocks;
-    // its beta partial sums land in part[0 .. fblocks) in a fixed order
-    const long long words = ((long long)a.nx * a.ny + 31) / 32;
-    const int fblocks = (int)((words + 255) / 256 < nblocks ? (words + 255) / 256 : nblocks);
+    cudaError_t e;
     switch (variant) {
-    case kLBGK: launch_adj_step_v<kLBGK, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
-#define KBC_ADJ_CASE(V)                                                                  \
-    case V:                                                                              \
-        launch_adj_step_v<V, C>(gp, li, lo, part, fixmask, nblocks, a, s);               \
-        if (fix) adj_fixup<V, C><<<fblocks, 256, 0, s>>>(gp, li, lo, part, fixmask, a); \
-        break;
-    KBC_ADJ_CASE(kA)
-    KBC_ADJ_CASE(kB)
-    KBC_ADJ_CASE(kC)
-    KBC_ADJ_CASE(kD)
-#undef KBC_ADJ_CASE
+    case kLBGK: e = launch_adj_step_v<kLBGK, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
+    case kA: e = launch_adj_step_v<kA, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
+    case kB: e = launch_adj_step_v<kB, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
+    case kC: e = launch_adj_step_v<kC, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
+    case kD: e = launch_adj_step_v<kD, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <class C>
