@@ -21,6 +21,7 @@
 
 #include <type_traits>
 
+#include "kbc_ff.cuh"
 #include "kbc_kernels.cuh"
 
 namespace kbc {
@@ -292,20 +293,28 @@ __device__ __forceinline__ bool collide_adjoint_pairs(const float (&d)[9], const
     return guarded;
 }
 
-// Returns true when the entropic denominator rho <dh|dh> is at or below
-// p.guard (entropic gamma only): there the derivative of gamma* with respect
-// to f, which carries 1 / <dh|dh>, is not resolved in the lane's precision,
-// and the caller re-evaluates the node in double (as the forward step does).
-template <int VAR, typename T>
-__device__ __forceinline__ bool collide_adjoint(const T (&d)[9], const T (&lam)[9],
-                                                const CollideParams<T>& p, T (&mu)[9],
-                                                T& beta_bar)
+// v_i . (x, y) without the products by 0 and 1 that double arithmetic would
+// have to carry out (0 x is not 0 for every x)
+__device__ __forceinline__ double along(int i, double x, double y)
 {
-    if constexpr (std::is_same<T, float>::value)
-        return collide_adjoint_pairs<VAR>(d, lam, p, mu, beta_bar);
-    bool guarded = false;
+    const int a = va(i), b = vb(i);
+    if (a == 0) return b == 0 ? 0.0 : (b > 0 ? y : -y);
+    if (b == 0) return a > 0 ? x : -x;
+    if (a == b) return a > 0 ? x + y : -(x + y);
+    return a > 0 ? x - y : -(x - y);
+}
+
+// Reverse collision of one node in double; the single-precision one is
+// collide_adjoint_pairs.  Bound by the FP64 pipe: about 540 FP64
+// instructions (820 with products by 0 and 1, separate products with
+// the weights and IEEE divisions).
+template <int VAR>
+__device__ __forceinline__ void collide_adjoint(const double (&d)[9], const double (&lam)[9],
+                                                const CollideParams<double>& p, double (&mu)[9],
+                                                double& beta_bar)
+{
+    using T = double;
     constexpr bool central = (VAR == kA || VAR == kB);
-    const T two_beta = p.two_beta;
     // ---------------------------------------------------------------- forward
     // pairwise sums (this order keeps the single-precision reverse closest
     // to the double one on long turbulent runs, where the linearised map
@@ -313,26 +322,23 @@ __device__ __forceinline__ bool collide_adjoint(const T (&d)[9], const T (&lam)[
     const T drho = ((d[0] + d[8]) + (d[2] + d[6])) + ((d[1] + d[7]) + (d[3] + d[5])) + d[4];
     const T jx = ((d[2] - d[0]) + (d[8] - d[6])) + (d[5] - d[3]);
     const T jy = ((d[6] - d[0]) + (d[8] - d[2])) + (d[7] - d[1]);
-    const T rho = T(1) + drho;
-    const T irho = rcp_fast(rho);
+    const T rho = 1.0 + drho;
+    const T irho = rcp_pos(rho);
     const T ux = jx * irho, uy = jy * irho;
-    const T usq15 = T(1.5) * (ux * ux + uy * uy);
-    T xi[9], P[9], df[9];
+    const T usq15 = 1.5 * (ux * ux + uy * uy);
+    T xi[9], P[9], x[9], df[9], dfb[9], Pb[9];
+    T uxb = 0.0, uyb = 0.0, bb = 0.0;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        xi[i] = T(va(i)) * ux + T(vb(i)) * uy;
-        P[i] = xi[i] * (T(3) + T(4.5) * xi[i]) - usq15;
-        df[i] = d[i] - T(wgt(i)) * (drho + rho * P[i]);
+        xi[i] = along(i, ux, uy);
+        P[i] = i == 4 ? -usq15 : fma(xi[i], fma(4.5, xi[i], 3.0), -usq15);
+        x[i] = fma(wgt(i), P[i], wgt(i));  // f^eq_i / rho
+        df[i] = fma(-wgt(i), fma(rho, P[i], drho), d[i]);
+        bb = fma(lam[i], df[i], bb);
+        dfb[i] = -p.two_beta * lam[i];
+        Pb[i] = 0.0;
     }
-    T dfb[9], Pb[9];
-    T uxb = T(0), uyb = T(0);
-    T bb = T(0);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        dfb[i] = -two_beta * lam[i];
-        Pb[i] = T(0);
-        bb -= T(2) * lam[i] * df[i];
-    }
+    bb *= -2.0;
     if constexpr (VAR != kLBGK) {
         const T corner = (df[0] + df[2]) + (df[6] + df[8]);
         const T m20 = corner + (df[3] + df[5]);
@@ -343,143 +349,191 @@ __device__ __forceinline__ bool collide_adjoint(const T (&d)[9], const T (&lam)[
             c20 = m20;
             c02 = m02;
         } else {
-            c20 = T(0.5) * (m20 - m02);
+            c20 = 0.5 * (m20 - m02);
             c02 = -c20;
         }
-        const T cx = central ? ux : T(0), cy = central ? uy : T(0);
-        const T e0x[3] = {T(0.5) * cx * (cx - T(1)), T(1) - cx * cx, T(0.5) * cx * (cx + T(1))};
-        const T e0y[3] = {T(0.5) * cy * (cy - T(1)), T(1) - cy * cy, T(0.5) * cy * (cy + T(1))};
-        const T e1x[3] = {cx - T(0.5), T(-2) * cx, cx + T(0.5)};
-        const T e1y[3] = {cy - T(0.5), T(-2) * cy, cy + T(0.5)};
-        const T e2[3] = {T(0.5), T(-1), T(0.5)};
-        T ds[9], dh[9], x[9], xi_inv[9], q[9];
-        T sh = T(0), hh = T(0);
+        // ds_(a,b) = c20 e2[a] e0y[b] + c02 e0x[a] e2[b] + m11 e1x[a] e1y[b],
+        // e0 = (c(c-1)/2, 1 - c^2, c(c+1)/2), e1 = (c - 1/2, -2c, c + 1/2),
+        // e2 = (1/2, -1, 1/2); the natural basis has c = 0
+        T e0x[3], e0y[3], e1x[3], e1y[3], ds[9];
+        if constexpr (central) {
+            const T hx = 0.5 * ux, hy = 0.5 * uy;
+            e0x[0] = fma(hx, ux, -hx);
+            e0x[1] = fma(-ux, ux, 1.0);
+            e0x[2] = fma(hx, ux, hx);
+            e0y[0] = fma(hy, uy, -hy);
+            e0y[1] = fma(-uy, uy, 1.0);
+            e0y[2] = fma(hy, uy, hy);
+            e1x[0] = ux - 0.5;
+            e1x[1] = -2.0 * ux;
+            e1x[2] = ux + 0.5;
+            e1y[0] = uy - 0.5;
+            e1y[1] = -2.0 * uy;
+            e1y[2] = uy + 0.5;
+            T Ay[3], Bx[3], Cx[3];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) x[i] = T(1) + P[i];
-        inv9(x, xi_inv);  // 1 / x_i
-        // ds_(a,b) = c20 e2[a] e0y[b] + c02 e0x[a] e2[b] + m11 e1x[a] e1y[b]
-        T Ay[3], Bx[3], Cx[3];
+            for (int k = 0; k < 3; ++k) {
+                Ay[k] = c20 * e0y[k];
+                Bx[k] = c02 * e0x[k];
+                Cx[k] = m11 * e1x[k];
+            }
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            Ay[k] = c20 * e0y[k];
-            Bx[k] = c02 * e0x[k];
-            Cx[k] = m11 * e1x[k];
+            for (int i = 0; i < 9; ++i) {
+                const int a = i % 3, b = i / 3;
+                const T ay = a == 1 ? -Ay[b] : 0.5 * Ay[b];  // e2[a] Ay[b]
+                ds[i] = fma(Cx[a], e1y[b], fma(b == 1 ? -1.0 : 0.5, Bx[a], ay));
+            }
+        } else {
+            const T q = 0.25 * m11;
+            ds[0] = ds[8] = q;
+            ds[2] = ds[6] = -q;
+            ds[3] = ds[5] = 0.5 * c20;
+            ds[1] = ds[7] = 0.5 * c02;
+            ds[4] = -(c20 + c02);
         }
+        // entropic weights q_i = rho / f^eq_i by Montgomery's inversion
+        T q[9], pre[9], t[9], v[9], dh[9];
+        pre[0] = x[0];
+#pragma unroll
+        for (int k = 1; k < 9; ++k) pre[k] = pre[k - 1] * x[k];
+        T inv = rcp_pos(pre[8]);
+#pragma unroll
+        for (int k = 8; k >= 1; --k) {
+            q[k] = inv * pre[k - 1];
+            inv *= x[k];
+        }
+        q[0] = inv;
+        T sh = 0.0, hh = 0.0;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            const int a = i % 3, b = i / 3;
-            ds[i] = Cx[a] * e1y[b] + (e2[a] * Ay[b] + e2[b] * Bx[a]);
             dh[i] = df[i] - ds[i];
-            q[i] = T(inv_wgt(i)) * xi_inv[i];
-            sh += ds[i] * dh[i] * q[i];
-            hh += dh[i] * dh[i] * q[i];
+            t[i] = dh[i] * q[i];
+            v[i] = ds[i] * q[i];
+            sh = fma(ds[i], t[i], sh);
+            hh = fma(dh[i], t[i], hh);
         }
-        T ch, R = T(0);
-        const bool has_h = hh > T(0);
-        guarded = !p.fixed && p.guard > T(0) && !(hh > p.guard);
-        const T ihh = has_h ? rcp_fast(hh) : T(0);
+        T ch, R = 0.0;
+        const bool has_h = hh > 0.0;
+        const T ihh = has_h ? rcp_pos(hh) : 0.0;
         if (p.fixed) {
             ch = p.ch_fixed;
         } else if (has_h) {
             R = sh * ihh;
-            ch = p.one_m_2beta * (T(1) + R);
+            ch = p.one_m_2beta * (1.0 + R);
         } else {
-            ch = T(0);
+            ch = 0.0;
         }
         // ---------------------------------------------------------- reverse
-        T dhb[9], dsb[9];
-        T chb = T(0);
+        T chb = 0.0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            dhb[i] = -ch * lam[i];
-            chb -= lam[i] * dh[i];
-        }
-        T Rb = T(0);
+        for (int i = 0; i < 9; ++i) chb = fma(-lam[i], dh[i], chb);
+        T Rb = 0.0;
         if (p.fixed) {
-            bb += chb * (p.gamma_fixed - T(2));
+            bb += chb * (p.gamma_fixed - 2.0);
         } else if (has_h) {
-            bb += chb * (T(-2) * (T(1) + R));
+            bb += chb * (-2.0 * (1.0 + R));
             Rb = chb * p.one_m_2beta;
         }
         const T shb = Rb * ihh;
         const T hhb = -Rb * R * ihh;
+        T dsb[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            dsb[i] = shb * dh[i] * q[i];
-            dhb[i] += shb * ds[i] * q[i] + T(2) * hhb * dh[i] * q[i];
-            const T qb = shb * ds[i] * dh[i] + hhb * dh[i] * dh[i];
-            Pb[i] -= qb * (q[i] * q[i]) * T(wgt(i));  // q_i / x_i = W_i q_i^2
-            dfb[i] += dhb[i];
-            dsb[i] -= dhb[i];
+            // with t = q dh, v = q ds: the adjoint of dh is shb v + 2 hhb t,
+            // that of the weight times dq/dP = -W q^2 is -W t (shb v + hhb t)
+            const T ht = hhb * t[i];
+            const T z = fma(shb, v[i], ht);
+            const T dhb = fma(-ch, lam[i], z + ht);
+            Pb[i] = (-wgt(i) * t[i]) * z;
+            dfb[i] += dhb;
+            dsb[i] = fma(shb, t[i], -dhb);
         }
         // reverse of ds through per-axis partial sums of D(a,b) = dsb[3b + a]:
         // S_b = sum_a e2[a] D, T_a = sum_b e2[b] D, U_a = sum_b e1y[b] D,
         // V_b = sum_a e1x[a] D
-        T S[3], Ta[3], U[3], V[3];
+        T S[3], Ta[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            S[k] = T(0.5) * (dsb[3 * k] + dsb[3 * k + 2]) - dsb[3 * k + 1];
-            Ta[k] = T(0.5) * (dsb[k] + dsb[6 + k]) - dsb[3 + k];
-            U[k] = e1y[0] * dsb[k] + e1y[1] * dsb[3 + k] + e1y[2] * dsb[6 + k];
-            V[k] = e1x[0] * dsb[3 * k] + e1x[1] * dsb[3 * k + 1] + e1x[2] * dsb[3 * k + 2];
+            S[k] = fma(0.5, dsb[3 * k] + dsb[3 * k + 2], -dsb[3 * k + 1]);
+            Ta[k] = fma(0.5, dsb[k] + dsb[6 + k], -dsb[3 + k]);
         }
-        const T c20b = e0y[0] * S[0] + e0y[1] * S[1] + e0y[2] * S[2];
-        const T c02b = e0x[0] * Ta[0] + e0x[1] * Ta[1] + e0x[2] * Ta[2];
-        const T m11b = e1x[0] * U[0] + e1x[1] * U[1] + e1x[2] * U[2];
-        T e0xb[3], e0yb[3], e1xb[3], e1yb[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            e0yb[k] = c20 * S[k];
-            e0xb[k] = c02 * Ta[k];
-            e1xb[k] = m11 * U[k];
-            e1yb[k] = m11 * V[k];
-        }
+        T c20b, c02b, m11b;
         if constexpr (central) {
-            // d e0(c)/dc = e1(c), d e1(c)/dc = (1, -2, 1)
+            T U[3], V[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                uxb += e0xb[k] * e1x[k] + e1xb[k] * (k == 1 ? T(-2) : T(1));
-                uyb += e0yb[k] * e1y[k] + e1yb[k] * (k == 1 ? T(-2) : T(1));
+                U[k] = fma(e1y[2], dsb[6 + k], fma(e1y[1], dsb[3 + k], e1y[0] * dsb[k]));
+                V[k] = fma(e1x[2], dsb[3 * k + 2], fma(e1x[1], dsb[3 * k + 1], e1x[0] * dsb[3 * k]));
             }
+            c20b = fma(e0y[2], S[2], fma(e0y[1], S[1], e0y[0] * S[0]));
+            c02b = fma(e0x[2], Ta[2], fma(e0x[1], Ta[1], e0x[0] * Ta[0]));
+            m11b = fma(e1x[2], U[2], fma(e1x[1], U[1], e1x[0] * U[0]));
+            // d e0(c)/dc = e1(c), d e1(c)/dc = (1, -2, 1)
+            uxb = fma(c02, fma(e1x[2], Ta[2], fma(e1x[1], Ta[1], e1x[0] * Ta[0])), m11 * ((U[0] + U[2]) - 2.0 * U[1]));
+            uyb = fma(c20, fma(e1y[2], S[2], fma(e1y[1], S[1], e1y[0] * S[0])), m11 * ((V[0] + V[2]) - 2.0 * V[1]));
+        } else {
+            c20b = S[1];
+            c02b = Ta[1];
+            m11b = 0.25 * ((dsb[0] + dsb[8]) - (dsb[2] + dsb[6]));
         }
         T m20b, m02b;
         if constexpr (VAR == kA || VAR == kC) {
             m20b = c20b;
             m02b = c02b;
         } else {
-            m20b = T(0.5) * (c20b - c02b);
+            m20b = 0.5 * (c20b - c02b);
             m02b = -m20b;
         }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const T a = T(va(i)), b = T(vb(i));
-            dfb[i] += a * a * m20b + b * b * m02b + a * b * m11b;
-        }
+        const T sb = m20b + m02b, sp = sb + m11b, sm = sb - m11b;
+        dfb[0] += sp;
+        dfb[8] += sp;
+        dfb[2] += sm;
+        dfb[6] += sm;
+        dfb[3] += m20b;
+        dfb[5] += m20b;
+        dfb[1] += m02b;
+        dfb[7] += m02b;
     }
     // ------------------------------------------------- equilibrium and moments
-    T drhob = T(0), usqb = T(0);
+    T drhob = 0.0, usqb = 0.0;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        // xi and P again from u (cheaper than keeping nine of each live)
-        const T xr = T(va(i)) * ux + T(vb(i)) * uy;
-        const T Pr = xr * (T(3) + T(4.5) * xr) - usq15;
         mu[i] = lam[i] + dfb[i];
-        drhob -= dfb[i] * T(wgt(i)) * (T(1) + Pr);
-        Pb[i] -= dfb[i] * T(wgt(i)) * rho;
+        drhob = fma(-dfb[i], x[i], drhob);
+        Pb[i] = fma(-dfb[i], wgt(i) * rho, Pb[i]);
         usqb -= Pb[i];
-        const T xib = Pb[i] * (T(3) + T(9) * xr);
-        uxb += T(va(i)) * xib;
-        uyb += T(vb(i)) * xib;
+        if (i == 4) continue;
+        const T xib = Pb[i] * fma(9.0, xi[i], 3.0);
+        if (va(i)) uxb += va(i) > 0 ? xib : -xib;
+        if (vb(i)) uyb += vb(i) > 0 ? xib : -xib;
     }
-    uxb += T(3) * ux * usqb;
-    uyb += T(3) * uy * usqb;
+    uxb = fma(3.0 * ux, usqb, uxb);
+    uyb = fma(3.0 * uy, usqb, uyb);
     const T jxb = uxb * irho, jyb = uyb * irho;
     const T irhob = uxb * jx + uyb * jy;
     drhob -= irhob * irho * irho;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) mu[i] += drhob + T(va(i)) * jxb + T(vb(i)) * jyb;
+    for (int i = 0; i < 9; ++i) mu[i] += i == 4 ? drhob : drhob + along(i, jxb, jyb);
     beta_bar = bb;
-    return guarded;
+}
+
+// The reverse collision in the storage's arithmetic type.  Returns true when
+// the entropic denominator rho <dh|dh> is at or below p.guard (entropic gamma
+// in single precision): there the derivative of gamma* with respect to f,
+// which carries 1 / <dh|dh>, is not resolved in that precision, and the caller
+// re-evaluates the node in double (as the forward step does).
+template <int VAR>
+__device__ __forceinline__ bool collide_reverse(const float (&d)[9], const float (&lam)[9],
+                                                const CollideParams<float>& p, float (&mu)[9], float& beta_bar)
+{
+    return collide_adjoint_pairs<VAR>(d, lam, p, mu, beta_bar);
+}
+template <int VAR>
+__device__ __forceinline__ bool collide_reverse(const double (&d)[9], const double (&lam)[9],
+                                                const CollideParams<double>& p, double (&mu)[9], double& beta_bar)
+{
+    collide_adjoint<VAR>(d, lam, p, mu, beta_bar);
+    return false;
 }
 
 // block-wide FP64 sum of v, added by thread 0 to *acc (fixed order)
@@ -551,7 +605,7 @@ __device__ __forceinline__ double adj_node(const typename C::S* __restrict__ g,
         lam[i] = ld_field(lam_in + (long long)i * a.plane + t);
     }
     T bbar;
-    const bool guarded = collide_adjoint<VAR>(d, lam, p, mu, bbar);
+    const bool guarded = collide_reverse<VAR>(d, lam, p, mu, bbar);
     if constexpr (!std::is_same<T, double>::value && VAR != kLBGK) {
         if (guarded) {
             atomicOr(fixmask + (n >> 5), 1u << (n & 31));
@@ -631,10 +685,12 @@ adj_fixup(const typename C::S* __restrict__ g, const typename C::T* __restrict__
     const long long total = (long long)a.nx * a.ny;
     const long long words = (total + 31) >> 5;
     double bsum = 0.0;
+    int any = 0;
     for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < words;
          w += (long long)gridDim.x * blockDim.x) {
         unsigned m = (unsigned)ld_count(reinterpret_cast<const int*>(fixmask + w));
         if (m == 0u) continue;
+        any = 1;
         fixmask[w] = 0u;
         while (m) {
             const int b = __ffs(m) - 1;
@@ -644,7 +700,7 @@ adj_fixup(const typename C::S* __restrict__ g, const typename C::T* __restrict__
             bsum += adj_node_f64<VAR, C>(g, lam_in, lam_out, n, x, y, a);
         }
     }
-    block_add(bsum, part + blockIdx.x);
+    if (__syncthreads_or(any)) block_add(bsum, part + blockIdx.x);  // adding 0 otherwise
 }
 
 // J of the final field and lambda^N = dJ/dg^N.  objective 0: kinetic energy

@@ -2,7 +2,7 @@
 // by per-thread asynchronous copies.
 //
 // Same arithmetic and outputs as adj_step (one node per thread over row
-// segments, collide_adjoint, the scatter of lambda^n to the pull sources,
+// segments, collide_reverse, the scatter of lambda^n to the pull sources,
 // the guard mask, the per-block beta sums).  While a thread computes its
 // node of one segment, the eighteen operands of its node in the next
 // segment (nine pulled forward-state values, nine of lambda^{n+1}) are
@@ -48,10 +48,10 @@ adj_step_async(const float* __restrict__ g, const float* __restrict__ lam_in,
     const int segs = nbx * a.ny;  // nx * ny < 2^31
     const int t = threadIdx.x;
     // each block takes a contiguous run of segments (fixed, so the beta sums
-    // keep their order), stepping row and column without a division
-    const int per = (segs + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int sg0 = (int)blockIdx.x * per;
-    const int sg1 = sg0 + per < segs ? sg0 + per : segs;
+    // keep their order; runs differ by one segment at most), stepping row and
+    // column without a division
+    const int sg0 = (int)((long long)segs * blockIdx.x / gridDim.x);
+    const int sg1 = (int)((long long)segs * (blockIdx.x + 1) / gridDim.x);
     // Offset of population i's pull source from node n: plane, source row
     // (y - b, periodic: dn / up for b = +1 / -1) and source column (x - a:
     // -a except at the row ends, where cl / cr wrap).  In a segment away from
@@ -118,7 +118,7 @@ adj_step_async(const float* __restrict__ g, const float* __restrict__ lam_in,
         }
         float bbar;
         const long long n = (long long)yc * a.nx + x;
-        const bool guarded = collide_adjoint<VAR>(d, lam, p, mu, bbar);
+        const bool guarded = collide_reverse<VAR>(d, lam, p, mu, bbar);
         if constexpr (VAR != kLBGK) {
             if (guarded) {
                 atomicOr(fixmask + (n >> 5), 1u << (n & 31));

@@ -1285,7 +1285,7 @@ int kbc_adjoint(kbc_handle h, const double* rho0, const double* u0, int nsteps, 
                         cudaError_t ec = by_codec(h->dtype, [&](auto c) {
                             using C = decltype(c);
                             return launch_adj_step<C>(h->variant, states[t - n0], lam[l], lam[l ^ 1],
-                                                      part + nb, fixmask, nb, ar, cs);
+                                                      part + nb, fixmask, nb, ar, cs, h->num_sms);
                         });
                         if (ec != cudaSuccess) return false;
                     }
@@ -1303,7 +1303,7 @@ int kbc_adjoint(kbc_handle h, const double* rho0, const double* u0, int nsteps, 
             e = by_codec(h->dtype, [&](auto c) {
                 using C = decltype(c);
                 return launch_adj_step<C>(h->variant, states[t - n0], lam[lc], lam[lc ^ 1],
-                                          part + nb, fixmask, nb, a, h->stream);
+                                          part + nb, fixmask, nb, a, h->stream, h->num_sms);
             });
             if (e != cudaSuccess) return cuda_fail(h, e, "adjoint step");
             lc ^= 1;

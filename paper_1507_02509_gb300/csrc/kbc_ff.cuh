@@ -4,7 +4,8 @@
 // however many of its lanes are active (measured: 64.1 cycles per DFMA with 1
 // to 32 active lanes, one warp per scheduler; conversions between 64-bit and
 // 32-bit types 81 to 89), against one cycle for an FP32 or integer
-// instruction.  Three tools follow.
+// instruction.  Two tools follow (and rcp_pos in kbc_lattice.cuh, a double
+// reciprocal by three fused multiply-adds).
 //
 // * FF<L>: an unevaluated sum of two floats (Dekker's and Knuth's error-free
 //   transformations), 48 bits, in the one-node lane Lf or the packed lane
@@ -14,8 +15,6 @@
 //   stored values are those of the double computation, always.
 // * Fixed sums: the nine stored populations as integers in one common unit,
 //   exact, so that rho and j are exact integer sums, rounded once.
-// * rcp_pos: a double reciprocal from the single-precision one and three
-//   double fused multiply-adds.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -116,22 +115,37 @@ __device__ __forceinline__ void round_sure(float s, float t, float err, unsigned
     }
 }
 
-// 1 / x in double, x > 0: the single-precision reciprocal y of the leading
-// bits (relative error below 2^-21), then y (1 + e + e^2) with the residual
-// e = 1 - x y, whose remainder e^3 is below the last bit.  Three FP64
-// instructions; the IEEE division takes about nine.
-__device__ __forceinline__ double rcp_pos(double x)
-{
-    const unsigned H = (unsigned)__double2hiint(x);
-    const unsigned e = H >> 20;
-    if (e - 923u >= 200u) return 1.0 / x;  // outside 2^-100 .. 2^100, negative or not finite
-    const float xf = __uint_as_float(((e - 896u) << 23) |
-                                     (__funnelshift_l((unsigned)__double2loint(x), H, 3) & 0x7fffffu));
-    const unsigned yb = __float_as_uint(__fdividef(1.0f, xf));
-    const double y = __hiloint2double((int)((yb >> 3) + 0x38000000u), (int)(yb << 29));
-    const double r = __fma_rn(-x, y, 1.0);
-    return __fma_rn(y, __fma_rn(r, r, r), y);
-}
+// Logarithms of 1 + x near 1 with eight FP64 instructions (the library's
+// log1p takes about thirty): the nearest multiple m of 1/128 from a table
+// {m, 1 / (1 + m), ln(1 + m)}, then ln(1 + r), r = (x - m) / (1 + m), as the
+// Taylor series to r^7, of which r^5 (1/5 - r/6 + r^2/7), 2^-28 of the whole,
+// needs no more than single precision.  For |x| < 1/2; the table is filled
+// by the kernel that uses it.
+struct LogTable {
+    static constexpr int kHalf = 64;
+    double m[2 * kHalf + 1], c[2 * kHalf + 1], l[2 * kHalf + 1];
+    __device__ __forceinline__ void fill()
+    {
+        for (int k = threadIdx.x; k <= 2 * kHalf; k += blockDim.x) {
+            m[k] = (double)(k - kHalf) * (0.5 / kHalf);
+            c[k] = 1.0 / (1.0 + m[k]);
+            l[k] = log1p(m[k]);
+        }
+    }
+    // x in double and rounded to float (to about 2^-20 of itself)
+    __device__ __forceinline__ double log1p_near(double x, float xf) const
+    {
+        const int k = __float2int_rn(xf * (2.0f * kHalf)) + kHalf;
+        const double r = (x - m[k]) * c[k];
+        const float mf = (float)(k - kHalf) * (0.5f / kHalf);
+        const float rf = (xf - mf) * __fdividef(1.0f, 1.0f + mf);
+        const float g = __fmaf_rn(rf, __fmaf_rn(rf, 1.0f / 7.0f, -1.0f / 6.0f), 0.2f);
+        double h = __fma_rn(r, widen_normal(g), -0.25);
+        h = __fma_rn(r, h, 1.0 / 3.0);
+        h = __fma_rn(r, h, -0.5);
+        return l[k] + __fma_rn(r * r, h, r);
+    }
+};
 
 // Exact sums over the nine stored populations as 64-bit integers: with
 // the unit double(unit) they are drho = rho - 1, jx and jy.  A value enters

@@ -677,9 +677,11 @@ __global__ void set_populations(const double* __restrict__ f, typename C::S* __r
     const long long total = (long long)a.nx * a.ny;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total;
          n += (long long)gridDim.x * blockDim.x) {
+        double v[9];  // all loads first: the conversions branch
 #pragma unroll
-        for (int i = 0; i < 9; ++i)
-            dst[(long long)i * a.plane + n] = C::from_f64(f[(long long)i * total + n] - wgt(i), i, a.cs);
+        for (int i = 0; i < 9; ++i) v[i] = f[(long long)i * total + n];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = C::from_f64(v[i] - wgt(i), i, a.cs);
     }
 }
 
@@ -690,9 +692,11 @@ __global__ void get_populations(const typename C::S* __restrict__ src, double* _
     const long long total = (long long)a.nx * a.ny;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total;
          n += (long long)gridDim.x * blockDim.x) {
+        typename C::S v[9];  // all loads first: the conversions branch
 #pragma unroll
-        for (int i = 0; i < 9; ++i)
-            f[(long long)i * total + n] = C::to_f64(src[(long long)i * a.plane + n], i, a.cs) + wgt(i);
+        for (int i = 0; i < 9; ++i) v[i] = src[(long long)i * a.plane + n];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[(long long)i * total + n] = C::to_f64(v[i], i, a.cs) + wgt(i);
     }
 }
 
@@ -779,13 +783,15 @@ moments(const typename C::S* __restrict__ src, double* __restrict__ rho,
 constexpr int kDiagParts = 11;
 constexpr int kDiagBlock = 256;
 
-// Welford's running update of (count n, mean m, M2 q) with one value x.
-__device__ __forceinline__ void welford_add(double& n, double& m, double& q, double x)
+// Welford's running update of mean m and M2 q with one value x, rn = 1 / n
+// with n the count including x.  The counts of both quantities of a thread
+// are the same, so one reciprocal (rcp_pos) serves both; with a division
+// each they took a tenth of the kernels' FP64 instructions.
+__device__ __forceinline__ void welford_add(double rn, double& m, double& q, double x)
 {
-    n += 1.0;
     const double d = x - m;
-    m += d / n;
-    q += d * (x - m);
+    m = __fma_rn(d, rn, m);
+    q = __fma_rn(d, x - m, q);
 }
 
 // Chan, Golub and LeVeque's combination of two partial (n, m, q) sets: the
@@ -873,18 +879,22 @@ diag_partial(const typename C::S* __restrict__ src, double* __restrict__ part, S
             const double ke = 0.5 * (ux * ux + uy * uy);
             const double w = 0.5 * (suy[cy][cx + 1] - suy[cy][cx - 1]) - 0.5 * (sux[cy + 1][cx] - sux[cy - 1][cx]);
             const double zz = 0.5 * w * w;
-            double cnt = acc[3];
-            welford_add(cnt, acc[4], acc[5], ke);
-            welford_add(acc[3], acc[6], acc[7], zz);
+            acc[3] += 1.0;
+            const double rn = rcp_pos(acc[3]);
+            welford_add(rn, acc[4], acc[5], ke);
+            welford_add(rn, acc[6], acc[7], zz);
+            const int xl = x == 0 ? a.nx - 1 : x - 1, xr = x + 1 == a.nx ? 0 : x + 1;
+            const int ym = pull_row(y - 1, a), yp = pull_row(y + 1, a);
+            typename C::S raw[9];
             double f[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                const int ai = i % 3 - 1, bi = i / 3 - 1;
-                int sx = x - ai, sy = y - bi;
-                sx = sx < 0 ? sx + a.nx : (sx >= a.nx ? sx - a.nx : sx);
-                sy = pull_row(sy, a);
-                f[i] = C::to_f64(src[(long long)i * a.plane + (long long)sy * a.nx + sx], i, a.cs);
+                const int sy = vb(i) == 1 ? ym : (vb(i) == -1 ? yp : y);
+                const int sx = va(i) == 1 ? xl : (va(i) == -1 ? xr : x);
+                raw[i] = src[(long long)i * a.plane + (long long)sy * a.nx + sx];
             }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = C::to_f64(raw[i], i, a.cs);
             double rr;
             bool hit;
             const double g = collide_node<VAR>(f, p, rr, hit);
@@ -929,6 +939,8 @@ diag_ext_partial(const typename C::S* __restrict__ src, double* __restrict__ par
     // u on the tile with a two-node halo, w on the tile with a one-node halo
     constexpr int UW = kTileW + 4, UH = kTileH + 4, WW = kTileW + 2, WH = kTileH + 2;
     __shared__ double sux[UH][UW], suy[UH][UW], sw[WH][WW];
+    __shared__ LogTable logs;
+    logs.fill();
     double acc[kDiagExtParts] = {0, 0, 0, 0, 0};  // n, mean and M2 of P, of s
     const int ntx = (a.nx + kTileW - 1) / kTileW, nty = (a.ny + kTileH - 1) / kTileH;
     const long long ntiles = (long long)ntx * nty;
@@ -957,15 +969,34 @@ diag_ext_partial(const typename C::S* __restrict__ src, double* __restrict__ par
             const double wy = 0.5 * (sw[cy + 1][cx] - sw[cy - 1][cx]);
             const double pp = 0.5 * (wx * wx + wy * wy);
             const long long n = (long long)y * a.nx + x;
-            double se = 0.0;
+            // s = -sum W_i (1 + x_i) ln(1 + x_i), x_i = d_i / W_i, by weight class
+            typename C::S raw[9];
+            double xs[9];
+            float xf[9];
+            bool near = true;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) raw[i] = src[(long long)i * a.plane + n];
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                const double d = C::to_f64(src[(long long)i * a.plane + n], i, a.cs);
-                se -= (wgt(i) + d) * log1p(d * inv_wgt(i));
+                xs[i] = C::to_f64(raw[i], i, a.cs) * inv_wgt(i);
+                xf[i] = leading(xs[i]);
+                near &= fabsf(xf[i]) < 0.5f;
             }
-            double cnt = acc[0];
-            welford_add(cnt, acc[1], acc[2], pp);
-            welford_add(acc[0], acc[3], acc[4], se);
+            double se = 0.0;
+            if (near) {
+                double sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+                for (int i = 0; i < 9; ++i)
+                    sum[wclass(i)] = __fma_rn(1.0 + xs[i], logs.log1p_near(xs[i], xf[i]), sum[wclass(i)]);
+                se = -__fma_rn(wgt(0), sum[0], __fma_rn(wgt(1), sum[1], wgt(4) * sum[2]));
+            } else {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) se -= wgt(i) * (1.0 + xs[i]) * log1p(xs[i]);
+            }
+            acc[0] += 1.0;
+            const double rn = rcp_pos(acc[0]);
+            welford_add(rn, acc[1], acc[2], pp);
+            welford_add(rn, acc[3], acc[4], se);
         }
     }
     __shared__ double sm[kDiagExtParts][kDiagBlock];

@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <type_traits>
 
+#include "kbc_lattice.cuh"
+
 namespace kbc {
 
 struct Lf {
@@ -51,12 +53,12 @@ __device__ __forceinline__ Ld operator-(Ld a, Ld b) { return Ld(__dsub_rn(a.v, b
 __device__ __forceinline__ Ld operator*(Ld a, Ld b) { return Ld(__dmul_rn(a.v, b.v)); }
 __device__ __forceinline__ Ld operator-(Ld a) { return Ld(-a.v); }
 __device__ __forceinline__ Ld fmaL(Ld a, Ld b, Ld c) { return Ld(__fma_rn(a.v, b.v, c.v)); }
-__device__ __forceinline__ Ld rcp_fast(Ld x) { return Ld(__drcp_rn(x.v)); }
-// a / b as a times the correctly rounded reciprocal of b (two roundings; in
-// the double collision it forms gamma*'s ratio <ds|dh> / <dh|dh>): 1.1% more
-// FP64 KBC B throughput than the correctly rounded quotient on GB300, whose
-// FP64 pipe bounds that path
-__device__ __forceinline__ Ld ratio(Ld a, Ld b) { return Ld(__dmul_rn(a.v, __drcp_rn(b.v))); }
+__device__ __forceinline__ Ld rcp_fast(Ld x) { return Ld(rcp_pos(x.v)); }
+// a / b as a times the reciprocal of b (in the double collision it forms
+// gamma*'s ratio <ds|dh> / <dh|dh>).  rcp_pos for this and for 1 / rho instead
+// of the correctly rounded reciprocal: 201 -> 189 FP64 instructions a node of
+// the step, whose FP64 pipe is the bound (1024^2 B 384 -> 362 us).
+__device__ __forceinline__ Ld ratio(Ld a, Ld b) { return Ld(__dmul_rn(a.v, rcp_pos(b.v))); }
 __device__ __forceinline__ unsigned gt_mask(Ld a, Ld b) { return a.v > b.v ? 1u : 0u; }
 __device__ __forceinline__ unsigned finite_mask(Ld a) { return isfinite(a.v) ? 1u : 0u; }
 __device__ __forceinline__ Ld select(unsigned m, Ld a, Ld b) { return (m & 1u) ? a : b; }

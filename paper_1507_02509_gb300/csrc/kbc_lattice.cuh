@@ -34,6 +34,84 @@ __host__ __device__ constexpr int wclass(int i)
     return (va(i) != 0 && vb(i) != 0) ? 0 : (va(i) == 0 && vb(i) == 0) ? 2 : 1;
 }
 
+// The conversion instructions between 32 and 64 bits take as long as an FP64
+// one, also where they are predicated off.  Out of line, so that the branches
+// below, which hardly any value takes, stay branches.
+static __device__ __noinline__ double cvt_f64(float v) { return (double)v; }
+static __device__ __noinline__ float cvt_f32(double v) { return __double2float_rn(v); }
+
+// A float as a double by integer operations; zeros included, subnormal,
+// infinite and NaN values by the instruction.
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned b = __float_as_uint(v), e = (b >> 23) & 0xffu;
+    if (e - 1u >= 254u && (b << 1) != 0u) return cvt_f64(v);
+    const unsigned m = e == 0u ? 0u : ((b & 0x7fffffffu) >> 3) + 0x38000000u;
+    return __hiloint2double((int)(m | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// the same for a positive normal float
+__device__ __forceinline__ double widen_normal(float v)
+{
+    const unsigned b = __float_as_uint(v);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+// A double rounded to the nearest float, ties to even: the truncated bits
+// plus the rounding, which may carry into the exponent.  Outside the normal
+// floats (and for zero) the instruction.
+__device__ __forceinline__ float narrow(double v)
+{
+    const unsigned H = (unsigned)__double2hiint(v), B = (unsigned)__double2loint(v);
+    const unsigned e = (H >> 20) & 0x7ffu;
+    if (e - 897u >= 254u) return cvt_f32(v);
+    const unsigned t = ((e - 896u) << 23) | (__funnelshift_l(B, H, 3) & 0x7fffffu), r = B & 0x1fffffffu;
+    const unsigned up = (r + (t & 1u)) > 0x10000000u ? 1u : 0u;
+    return __uint_as_float((t + up) | (H & 0x80000000u));
+}
+
+// A double rounded to a float whose last bit is set when the value is not
+// exact (round to odd), from which rounding on to half gives the nearest half.
+__device__ __forceinline__ float narrow_odd(double v)
+{
+    const unsigned H = (unsigned)__double2hiint(v), B = (unsigned)__double2loint(v);
+    const unsigned e = (H >> 20) & 0x7ffu;
+    if (e < 897u) return __uint_as_float(H & 0x80000000u);  // a half of zero
+    if (e >= 1151u) return cvt_f32(v);
+    const unsigned t = ((e - 896u) << 23) | (__funnelshift_l(B, H, 3) & 0x7fffffu);
+    return __uint_as_float(t | ((B & 0x1fffffffu) ? 1u : 0u) | (H & 0x80000000u));
+}
+
+// The leading 24 bits of a double as a float (truncated), for magnitudes in
+// 2^-74 .. 8; 0 below, NaN outside.
+__device__ __forceinline__ float leading(double v)
+{
+    const unsigned H = (unsigned)__double2hiint(v), e = (H >> 20) & 0x7ffu;
+    const unsigned f = (__funnelshift_l((unsigned)__double2loint(v), H, 3) & 0x7fffffu) | ((e - 896u) << 23);
+    return e < 949u ? 0.0f : e > 1025u ? __uint_as_float(0x7fffffffu) : __uint_as_float(f | (H & 0x80000000u));
+}
+
+// out of line for the same reason
+static __device__ __noinline__ double divide_one(double x) { return 1.0 / x; }
+
+// 1 / x in double for positive normal x (others by the IEEE division): with
+// x = m 2^k, 1 <= m < 2, the single-precision reciprocal y of m's leading bits
+// (relative error below 2^-21), then y (1 + r + r^2) with the residual
+// r = 1 - m y, whose remainder r^3 is below the last bit.  Three FP64
+// instructions; the IEEE division takes about nine.
+__device__ __forceinline__ double rcp_pos(double x)
+{
+    const unsigned H = (unsigned)__double2hiint(x), B = (unsigned)__double2loint(x);
+    const unsigned e = H >> 20;
+    if (e - 1u >= 2044u) return divide_one(x);  // not a positive normal with a normal reciprocal
+    const float mf = __uint_as_float(0x3f800000u | (__funnelshift_l(B, H, 3) & 0x7fffffu));
+    const double m = __hiloint2double((int)((H & 0xfffffu) | 0x3ff00000u), (int)B);
+    const double y = widen_normal(__fdividef(1.0f, mf));
+    const double r = __fma_rn(-m, y, 1.0);
+    const double z = __fma_rn(y, __fma_rn(r, r, r), y);  // in (1/2, 1]
+    return __hiloint2double(__double2hiint(z) + (int)((1023u - e) << 20), __double2loint(z));
+}
+
 // Scale of the half-precision encoding (unused by the other codecs): S and,
 // per weight class, the decode factor W/S, rounded once on the host so that
 // the kernels take it from the parameter bank instead of forming it per
@@ -93,8 +171,8 @@ struct CodecF32 {
     __device__ __forceinline__ static T decode(S s, int, const CodecScale&) { return s; }
     __device__ __forceinline__ static T load(S s, int, const CodecScale&) { return s; }
     __device__ __forceinline__ static S store(T d, int, const CodecScale&) { return d; }
-    __device__ __forceinline__ static double to_f64(S s, int, const CodecScale&) { return (double)s; }
-    __device__ __forceinline__ static S from_f64(double d, int, const CodecScale&) { return __double2float_rn(d); }
+    __device__ __forceinline__ static double to_f64(S s, int, const CodecScale&) { return widen(s); }
+    __device__ __forceinline__ static S from_f64(double d, int, const CodecScale&) { return narrow(d); }
 };
 
 // (f - W)/W * S in IEEE half (stored as its 16-bit pattern), arithmetic in
@@ -126,11 +204,11 @@ struct CodecF16 {
     }
     __device__ __forceinline__ static double to_f64(S s, int i, const CodecScale& c)
     {
-        return (double)__half2float(__ushort_as_half(s)) * (wgt(i) * (double)c.inv_scale);
+        return widen(__half2float(__ushort_as_half(s))) * (wgt(i) * (double)c.inv_scale);
     }
     __device__ __forceinline__ static S from_f64(double d, int i, const CodecScale& c)
     {
-        return __half_as_ushort(__double2half(d * (inv_wgt(i) * (double)c.scale)));
+        return __half_as_ushort(__float2half_rn(narrow_odd(d * (inv_wgt(i) * (double)c.scale))));
     }
 };
 

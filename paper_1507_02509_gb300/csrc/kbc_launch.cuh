@@ -228,6 +228,7 @@ cudaError_t launch_diag_ext(const void* src, double* part, int nblocks, double* 
 
 // ---------------------------------------------------------------- adjoint
 
+// Blocks of the objective and of the reverse steps, one beta partial sum each.
 inline int adj_blocks(long long total, int num_sms) { return grid_for(total, 256, num_sms, 8); }
 
 // One reverse step: FP32 storage prefetches each thread's operands by
@@ -235,12 +236,18 @@ inline int adj_blocks(long long total, int num_sms) { return grid_for(total, 256
 // by node (adj_step).
 template <int VAR, class C>
 cudaError_t launch_adj_step_v(const typename C::S* g, const typename C::T* li, typename C::T* lo,
-                              double* part, unsigned* fixmask, int nblocks, const StepArgs& a, cudaStream_t s)
+                              double* part, unsigned* fixmask, int nblocks, const StepArgs& a, cudaStream_t s,
+                              int num_sms)
 {
     cudaError_t e;
-    if constexpr (std::is_same<C, CodecF32>::value)
-        e = launch_chained(adj_step_async<VAR>, nblocks, kAdjBlock, 0, s, g, li, lo, part, fixmask, a);
-    else
+    if constexpr (std::is_same<C, CodecF32>::value) {
+        // one wave of resident blocks (adj_min_blocks per SM), each with its
+        // share of the segments: a second, partly filled wave would start
+        // its prefetch pipeline anew
+        const int wave = num_sms * adj_min_blocks<VAR, float>();
+        e = launch_chained(adj_step_async<VAR>, nblocks < wave ? nblocks : wave, kAdjBlock, 0, s, g, li, lo, part,
+                           fixmask, a);
+    } else
         e = launch_chained(adj_step<VAR, C>, nblocks, kAdjBlock, 0, s, g, li, lo, part, fixmask, a);
     if constexpr (VAR != kLBGK && !std::is_same<typename C::T, double>::value) {
         // the double redo scans one mask word per thread: a grid sized to the
@@ -257,7 +264,7 @@ cudaError_t launch_adj_step_v(const typename C::S* g, const typename C::T* li, t
 template <class C>
 cudaError_t launch_adj_step(int variant, const void* g, const void* lam_in, void* lam_out,
                             double* part, unsigned* fixmask, int nblocks, const StepArgs& a,
-                            cudaStream_t s)
+                            cudaStream_t s, int num_sms)
 {
     using S = typename C::S;
     using T = typename C::T;
@@ -266,11 +273,11 @@ cudaError_t launch_adj_step(int variant, const void* g, const void* lam_in, void
     T* lo = static_cast<T*>(lam_out);
     cudaError_t e;
     switch (variant) {
-    case kLBGK: e = launch_adj_step_v<kLBGK, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
-    case kA: e = launch_adj_step_v<kA, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
-    case kB: e = launch_adj_step_v<kB, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
-    case kC: e = launch_adj_step_v<kC, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
-    case kD: e = launch_adj_step_v<kD, C>(gp, li, lo, part, fixmask, nblocks, a, s); break;
+    case kLBGK: e = launch_adj_step_v<kLBGK, C>(gp, li, lo, part, fixmask, nblocks, a, s, num_sms); break;
+    case kA: e = launch_adj_step_v<kA, C>(gp, li, lo, part, fixmask, nblocks, a, s, num_sms); break;
+    case kB: e = launch_adj_step_v<kB, C>(gp, li, lo, part, fixmask, nblocks, a, s, num_sms); break;
+    case kC: e = launch_adj_step_v<kC, C>(gp, li, lo, part, fixmask, nblocks, a, s, num_sms); break;
+    case kD: e = launch_adj_step_v<kD, C>(gp, li, lo, part, fixmask, nblocks, a, s, num_sms); break;
     default: return cudaErrorInvalidValue;
     }
     return e == cudaSuccess ? cudaGetLastError() : e;
@@ -317,7 +324,7 @@ cudaError_t launch_adj_grad_u0(const double* rho0, const double* ux0, const doub
                                                    const StepArgs&, cudaStream_t);            \
     extern template cudaError_t launch_adj_step<C>(int, const void*, const void*, void*,      \
                                                    double*, unsigned*, int, const StepArgs&,  \
-                                                   cudaStream_t);                             \
+                                                   cudaStream_t, int);                        \
     extern template cudaError_t launch_adj_objective<C>(const void*, const double*,           \
                                                         const double*, int, void*, double*,   \
                                                         int, const StepArgs&, cudaStream_t);  \
@@ -343,7 +350,8 @@ cudaError_t launch_adj_grad_u0(const double* rho0, const double* ux0, const doub
     template cudaError_t launch_diag_ext<C>(const void*, double*, int, double*,               \
                                             const StepArgs&, cudaStream_t);                   \
     template cudaError_t launch_adj_step<C>(int, const void*, const void*, void*, double*,    \
-                                            unsigned*, int, const StepArgs&, cudaStream_t);   \
+                                            unsigned*, int, const StepArgs&, cudaStream_t,    \
+                                            int);                                             \
     template cudaError_t launch_adj_objective<C>(const void*, const double*, const double*,   \
                                                  int, void*, double*, int, const StepArgs&,   \
                                                  cudaStream_t);                               \
