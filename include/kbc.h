@@ -321,10 +321,12 @@ int kbc_diagnostics_ext(kbc_handle h, double* out);
  *   host or device; shells k >= nbins are left out (all fit when nbins >=
  *   round(n sqrt(2) / 2) + 1).  stream: CUDA stream (NULL: the legacy
  *   default stream); the call synchronises it before returning.
- * The FFT is cuFFT (a library step); the binning is this library's kernel.
+ * The FFT is cuFFT (a library step; its plans, which hold no device memory of
+ * the allocator, are kept for up to eight sizes); the binning is this
+ * library's kernel.
  * Its shell sums use atomic additions, so their last bits depend on the
  * order of the additions.  Device scratch (the velocity staging for host
- * input, the half spectrum, cuFFT's work area) comes from the allocator set
+ * input, the complex field, cuFFT's work area) comes from the allocator set
  * with kbc_set_allocator (default cudaMalloc) and is released before the
  * call returns.  Errors: KBC_ERR_ARG, KBC_ERR_NOMEM, KBC_ERR_CUDA (message:
  * kbc_last_error(NULL)). */

@@ -10,6 +10,7 @@
 #include <thread>
 #include <vector>
 
+#include <cudaTypedefs.h>
 #include <cufft.h>
 
 #include "../../include/kbc.h"
@@ -115,6 +116,141 @@ int kbc::handle_free_error(int code, const char* msg)
     return code;
 }
 
+unsigned long long kbc::current_context_id()
+{
+    static const PFN_cuCtxGetId_v12000 get_id = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        cudaGetLastError();
+        return ok ? reinterpret_cast<PFN_cuCtxGetId_v12000>(fn) : nullptr;
+    }();
+    unsigned long long id = 0;
+    if (!get_id || get_id(nullptr, &id) != CUDA_SUCCESS) return 0;
+    return id;
+}
+
+// Host resources kept between objects and calls, because making them costs
+// more than a small problem computes.  Both are bounded, handed out to one
+// owner at a time under a lock, and belong to the context they were made in.
+//
+// Pinned status words of the handles: 256 slots of one page (the first
+// pinned allocation of a process without one takes 230 us; creating and
+// destroying a handle 398 -> 165 us).
+namespace {
+
+struct FlagPool {
+    static constexpr int kSlots = 256, kInts = 4;
+    std::mutex mu;
+    int* page = nullptr;
+    unsigned long long ctx = 0;
+    bool used[kSlots] = {};
+
+    int* get()
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        const unsigned long long id = current_context_id();
+        if (id != 0 && (!page || ctx != id)) {  // another context's page went with it
+            page = nullptr;
+            if (cudaHostAlloc((void**)&page, kSlots * kInts * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+                cudaGetLastError();
+                page = nullptr;
+            }
+            ctx = id;
+            for (bool& u : used) u = false;
+        }
+        for (int k = 0; page && id == ctx && k < kSlots; ++k)
+            if (!used[k]) {
+                used[k] = true;
+                return page + k * kInts;
+            }
+        int* own = nullptr;
+        if (cudaHostAlloc((void**)&own, kInts * sizeof(int), cudaHostAllocDefault) != cudaSuccess) return nullptr;
+        return own;
+    }
+    // the caller has waited for every copy into it
+    void put(int* p)
+    {
+        if (!p) return;
+        std::lock_guard<std::mutex> lk(mu);
+        if (page && p >= page && p < page + kSlots * kInts) used[(p - page) / kInts] = false;
+        else cudaFreeHost(p);
+    }
+};
+FlagPool g_flags;
+
+// cuFFT plans of kbc_spectrum by size (making one takes 0.3 to 0.5 ms, more
+// than the transform of a 1024^2 field); the work area is the call's own.
+struct PlanPool {
+    static constexpr int kPlans = 8;
+    struct Entry {
+        cufftHandle plan = 0;
+        size_t work = 0;
+        int n = 0, device = -1;
+        unsigned long long ctx = 0, age = 0;
+        bool held = false;
+    };
+    std::mutex mu;
+    Entry e[kPlans];
+    unsigned long long clock = 0;
+
+    // a plan that nobody else uses until put(); false when cuFFT fails
+    bool get(int n, int device, Entry* out)
+    {
+        const unsigned long long id = current_context_id();
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            for (Entry& x : e)
+                if (x.held && id != 0 && x.n == n && x.device == device && x.ctx == id) {
+                    *out = x;
+                    x = Entry();
+                    return true;
+                }
+        }
+        Entry x;
+        if (cufftCreate(&x.plan) != CUFFT_SUCCESS) return false;
+        if (cufftSetAutoAllocation(x.plan, 0) != CUFFT_SUCCESS ||
+            cufftMakePlan2d(x.plan, n, n, CUFFT_Z2Z, &x.work) != CUFFT_SUCCESS) {
+            cufftDestroy(x.plan);
+            return false;
+        }
+        x.n = n;
+        x.device = device;
+        x.ctx = id;
+        *out = x;
+        return true;
+    }
+    // the caller has waited for the plan's work
+    void put(Entry x)
+    {
+        Entry old;
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            Entry* to = &e[0];
+            for (Entry& y : e) {
+                if (!y.held) {
+                    to = &y;
+                    break;
+                }
+                if (y.age < to->age) to = &y;
+            }
+            old = *to;
+            x.held = x.ctx != 0;
+            x.age = ++clock;
+            if (x.held) *to = x;
+            else old = x, old.held = true;
+        }
+        // the least recently used one makes room; one of a context that is
+        // gone went with it
+        if (old.held && (old.ctx == 0 || old.ctx == current_context_id())) cufftDestroy(old.plan);
+    }
+};
+PlanPool g_plans;
+
+}  // namespace
+
 // Row chunks of the host <-> device pipelines of kbc_init and kbc_moments;
 // staging below kPipeMinBytes uses one copy and one kernel.
 constexpr int kPipeChunks = 32;
@@ -153,12 +289,18 @@ struct kbc_ctx {
     unsigned config_version = 1;
     unsigned graph_version[4] = {0, 0, 0, 0};
     cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
+    // the same for the even number of steps below graph_steps that the last
+    // two calls ended with (short_len; captured when it is seen again)
+    int short_len = 0;
+    unsigned short_version[4] = {0, 0, 0, 0};
+    cudaGraphExec_t short_graph[4] = {nullptr, nullptr, nullptr, nullptr};
     cudaStream_t capture_stream = nullptr;
     // host <-> device pipelines: copies of one row chunk overlap the kernel
     // of the neighbouring chunk on this second stream, ordered by events
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t pipe_ev[kPipeChunks + 2] = {};
     cudaStream_t stream = nullptr;
+    bool restreamed = false;  // another stream was bound while there was work
     Allocator al;
     std::string err;
 };
@@ -342,58 +484,6 @@ static int step_into(kbc_handle h, const void* src, void* dst, cudaStream_t stre
     return KBC_OK;
 }
 
-static void drop_graphs(kbc_handle h)
-{
-    for (int k = 0; k < 4; ++k) {
-        if (h->graph[k]) cudaGraphExecDestroy(h->graph[k]);
-        h->graph[k] = nullptr;
-        h->graph_version[k] = 0;
-    }
-}
-
-// The instantiated graph of graph_steps steps starting from the current
-// (cur, fix_slot) parity, captured on a private stream; nullptr if capture
-// is not possible (the step then runs launch by launch).
-static cudaGraphExec_t step_graph(kbc_handle h)
-{
-    const int key = h->cur | (h->fix_slot << 1);
-    if (h->graph[key] && h->graph_version[key] == h->config_version) return h->graph[key];
-    if (h->graph[key]) {
-        cudaGraphExecDestroy(h->graph[key]);
-        h->graph[key] = nullptr;
-    }
-    if (!h->capture_stream &&
-        cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaGetLastError();
-        h->capture_stream = nullptr;
-        return nullptr;
-    }
-    const int slot0 = h->fix_slot;
-    if (cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    int c = h->cur;
-    bool ok = true;
-    for (int s = 0; s < h->graph_steps && ok; ++s) {
-        ok = step_into(h, h->buf[c], h->buf[c ^ 1], h->capture_stream, true) == KBC_OK;
-        c ^= 1;
-    }
-    cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(h->capture_stream, &g);
-    h->fix_slot = slot0;  // graph_steps is even: the replay returns to this parity
-    cudaGraphExec_t exec = nullptr;
-    if (ok && e == cudaSuccess && g && cudaGraphInstantiate(&exec, g, 0) == cudaSuccess) {
-        h->graph[key] = exec;
-        h->graph_version[key] = h->config_version;
-    } else {
-        exec = nullptr;
-    }
-    if (g) cudaGraphDestroy(g);
-    cudaGetLastError();
-    return exec;
-}
-
 // Instantiated graph of the work `issue(stream)` enqueues on the private
 // capture stream (returns false on a failed launch); nullptr when capture or
 // instantiation fails, with the handle's guard parity restored, so that the
@@ -422,6 +512,55 @@ static cudaGraphExec_t capture_work(kbc_handle h, F&& issue)
     }
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
+    return exec;
+}
+
+static void drop_short_graphs(kbc_handle h)
+{
+    bool any = false;
+    for (cudaGraphExec_t g : h->short_graph) any |= g != nullptr;
+    if (any) cudaStreamSynchronize(h->stream);  // the last replay may still run
+    for (int k = 0; k < 4; ++k) {
+        if (h->short_graph[k]) cudaGraphExecDestroy(h->short_graph[k]);
+        h->short_graph[k] = nullptr;
+        h->short_version[k] = 0;
+    }
+}
+
+static void drop_graphs(kbc_handle h)
+{
+    for (int k = 0; k < 4; ++k) {
+        if (h->graph[k]) cudaGraphExecDestroy(h->graph[k]);
+        h->graph[k] = nullptr;
+        h->graph_version[k] = 0;
+    }
+    drop_short_graphs(h);
+    h->short_len = 0;
+}
+
+// The instantiated graph of `steps` (even) steps starting from the current
+// (cur, fix_slot) parity, kept in slot[] while the configuration stays as it
+// is; nullptr if capture is not possible (the steps then run launch by launch).
+static cudaGraphExec_t step_graph(kbc_handle h, int steps, cudaGraphExec_t* slot, unsigned* version)
+{
+    const int key = h->cur | (h->fix_slot << 1);
+    if (slot[key] && version[key] == h->config_version) return slot[key];
+    if (slot[key]) {
+        cudaGraphExecDestroy(slot[key]);
+        slot[key] = nullptr;
+    }
+    const int slot0 = h->fix_slot;
+    cudaGraphExec_t exec = capture_work(h, [&](cudaStream_t cs) {
+        int c = h->cur;
+        for (int s = 0; s < steps; ++s, c ^= 1)
+            if (step_into(h, h->buf[c], h->buf[c ^ 1], cs, true) != KBC_OK) return false;
+        return true;
+    });
+    h->fix_slot = slot0;  // steps is even: the replay returns to this parity
+    if (exec) {
+        slot[key] = exec;
+        version[key] = h->config_version;
+    }
     return exec;
 }
 
@@ -668,10 +807,9 @@ static int create_common(int nx, int ny, int variant, double beta, int dtype, bo
         kbc_destroy(h);
         return fail(nullptr, KBC_ERR_NOMEM, "device allocation failed");
     }
-    e = cudaHostAlloc((void**)&h->flag_host, 4 * sizeof(int), cudaHostAllocDefault);
-    if (e != cudaSuccess) {
+    h->flag_host = g_flags.get();
+    if (!h->flag_host) {
         cudaGetLastError();
-        h->flag_host = nullptr;
         kbc_destroy(h);
         return fail(nullptr, KBC_ERR_CUDA, "pinned allocation failed");
     }
@@ -704,7 +842,9 @@ int kbc_destroy(kbc_handle h)
 {
     if (!h) return KBC_ERR_ARG;
     cudaSetDevice(h->device);
-    cudaStreamSynchronize(h->stream);
+    // every stream that may still write the handle's status words
+    if (h->restreamed) cudaDeviceSynchronize();
+    else cudaStreamSynchronize(h->stream);
     dev_free(h, h->alloc[0]);
     dev_free(h, h->alloc[1]);
     dev_free(h, h->fix);
@@ -712,7 +852,7 @@ int kbc_destroy(kbc_handle h)
     dev_free(h, h->diag_part);
     dev_free(h, h->diag_out);
     dev_free(h, h->stage);
-    if (h->flag_host) cudaFreeHost(h->flag_host);
+    g_flags.put(h->flag_host);
     drop_graphs(h);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
@@ -726,6 +866,7 @@ int kbc_destroy(kbc_handle h)
 int kbc_set_stream(kbc_handle h, void* stream)
 {
     if (!h) return KBC_ERR_ARG;
+    if (h->initialized && h->stream != static_cast<cudaStream_t>(stream)) h->restreamed = true;
     h->stream = static_cast<cudaStream_t>(stream);
     return KBC_OK;
 }
@@ -868,12 +1009,31 @@ int kbc_step(kbc_handle h, int nsteps)
                            cs != cudaStreamCaptureStatusNone;
     cudaGetLastError();
     if (h->graph_steps > 0 && nsteps >= h->graph_steps && !capturing) {
-        cudaGraphExec_t g = step_graph(h);
+        cudaGraphExec_t g = step_graph(h, h->graph_steps, h->graph, h->graph_version);
         if (g) {
             for (; done + h->graph_steps <= nsteps; done += h->graph_steps) {
                 cudaError_t e = cudaGraphLaunch(g, h->stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
             }
+        }
+    }
+    // The rest below graph_steps: programs that take a few steps between looks
+    // at the field ask for the same number again and again, and launching
+    // them one by one costs more than small grids compute (128^2, float C, ten
+    // steps: 20 launches, 56 us, against 25 us for the replay).  One call of a
+    // length launches directly, so that it does not pay for a capture.
+    const int rest = (nsteps - done) & ~1;
+    if (h->graph_steps > 0 && rest >= 4 && !capturing) {
+        if (rest == h->short_len) {
+            cudaGraphExec_t g = step_graph(h, rest, h->short_graph, h->short_version);
+            if (g) {
+                cudaError_t e = cudaGraphLaunch(g, h->stream);
+                if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
+                done += rest;
+            }
+        } else {
+            drop_short_graphs(h);
+            h->short_len = rest;
         }
     }
     for (int s = done; s < nsteps; ++s) {
@@ -1514,7 +1674,7 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
         cudaStream_t s;
         void* p[4] = {nullptr, nullptr, nullptr, nullptr};
         int k = 0;
-        cufftHandle plan = 0;
+        PlanPool::Entry fft;
         bool planned = false;
         void* get(size_t bytes)
         {
@@ -1531,7 +1691,7 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
         ~Scratch()
         {
             cudaStreamSynchronize(s);
-            if (planned) cufftDestroy(plan);
+            if (planned) g_plans.put(fft);
             for (int j = 0; j < k; ++j) {
                 if (al.release) al.release(p[j], (void*)s, al.user);
                 else cudaFree(p[j]);
@@ -1548,36 +1708,31 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "spectrum: upload");
         du = st;
     }
-    double2* uh = static_cast<double2*>(sc.get((size_t)n * (n / 2 + 1) * sizeof(double2)));
+    double2* uh = static_cast<double2*>(sc.get(nn * sizeof(double2)));
     double* acc = static_cast<double*>(sc.get(2 * (size_t)nbins * sizeof(double)));
     if (!uh || !acc) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: scratch allocation failed");
     // cuFFT (a library step) with its work area from the same allocator
-    size_t ws = 0;
-    if (cufftCreate(&sc.plan) != CUFFT_SUCCESS) return fail(nullptr, KBC_ERR_CUDA, "spectrum: cufftCreate");
-    sc.planned = true;
-    if (cufftSetAutoAllocation(sc.plan, 0) != CUFFT_SUCCESS ||
-        cufftMakePlan2d(sc.plan, n, n, CUFFT_D2Z, &ws) != CUFFT_SUCCESS)
-        return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT plan");
-    void* work = sc.get(ws);
-    if (!work) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: cuFFT work area allocation failed");
-    if (cufftSetWorkArea(sc.plan, work) != CUFFT_SUCCESS || cufftSetStream(sc.plan, s) != CUFFT_SUCCESS)
-        return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT work area / stream");
-    cudaError_t e = cudaMemsetAsync(acc, 0, (size_t)nbins * sizeof(double), s);
-    if (e != cudaSuccess) return cuda_fail(nullptr, e, "spectrum: memset");
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (!g_plans.get(n, dev, &sc.fft)) return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT plan");
+    sc.planned = true;
+    void* work = sc.get(sc.fft.work);
+    if (!work) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: cuFFT work area allocation failed");
+    if (cufftSetWorkArea(sc.fft.plan, work) != CUFFT_SUCCESS || cufftSetStream(sc.fft.plan, s) != CUFFT_SUCCESS)
+        return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT work area / stream");
+    cudaError_t e = cudaMemsetAsync(acc, 0, (size_t)nbins * sizeof(double), s);
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "spectrum: memset");
     const size_t smem = (size_t)nbins * sizeof(double);
     const int use_smem = smem <= (size_t)160 * 1024 ? 1 : 0;
     if (use_smem && smem > 48 * 1024)
         cudaFuncSetAttribute(spectrum_bin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const double scale = 1.0 / ((double)nn * (double)nn);
-    for (int c = 0; c < 2; ++c) {
-        if (cufftExecD2Z(sc.plan, const_cast<double*>(du) + c * nn, reinterpret_cast<cufftDoubleComplex*>(uh)) !=
-            CUFFT_SUCCESS)
-            return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT execution");
-        spectrum_bin<<<sms * 4, 256, use_smem ? smem : 0, s>>>(uh, n, nbins, scale, acc, use_smem);
-    }
+    spectrum_pack<<<sms * 8, 256, 0, s>>>(du, (long long)nn, uh);
+    if (cufftExecZ2Z(sc.fft.plan, reinterpret_cast<cufftDoubleComplex*>(uh), reinterpret_cast<cufftDoubleComplex*>(uh),
+                     CUFFT_FORWARD) != CUFFT_SUCCESS)
+        return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT execution");
+    spectrum_bin<<<sms * 4, 256, use_smem ? smem : 0, s>>>(uh, n, nbins, scale, acc, use_smem);
     spectrum_enstrophy<<<(nbins + 255) / 256, 256, 0, s>>>(acc, acc + nbins, nbins, n);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(E, acc, (size_t)nbins * sizeof(double), cudaMemcpyDefault, s);

@@ -14,6 +14,10 @@
 
 namespace kbc {
 
+// Unique id of the current context, which tells one created after
+// cudaDeviceReset from the one before; 0 when it cannot be had.
+unsigned long long current_context_id();
+
 // rows: vectorised row kernel (nx % (32 * kVec) == 0); nodes: any width;
 // bulk: persistent bulk-copy kernel (nx % kTmaTile == 0, F32/F16)
 enum class StepKind { rows, nodes, bulk };

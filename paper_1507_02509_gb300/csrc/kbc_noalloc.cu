@@ -13,8 +13,6 @@
 #include <mutex>
 #include <thread>
 
-#include <cudaTypedefs.h>
-
 #include "../../include/kbc.h"
 #include "kbc_launch.cuh"
 
@@ -40,27 +38,6 @@ __device__ __align__(256) double g_noalloc_scratch[kMaxBlocks * kDiagParts + 32]
 std::mutex g_mu;
 double* g_scratch_addr[kMaxDevices] = {};
 unsigned long long g_scratch_ctx[kMaxDevices] = {};
-
-// Unique id of the current context (0 when it cannot be had: the address is
-// then looked up on every call instead of cached).
-unsigned long long current_context_id()
-{
-    static PFN_cuCtxGetId_v12000 get_id = nullptr;
-    static bool looked_up = false;
-    if (!looked_up) {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<PFN_cuCtxGetId_v12000>(fn);
-        cudaGetLastError();
-        looked_up = true;
-    }
-    unsigned long long id = 0;
-    if (!get_id || get_id(nullptr, &id) != CUDA_SUCCESS) return 0;
-    return id;
-}
 
 }  // namespace
 }  // namespace kbc
@@ -97,7 +74,7 @@ extern "C" int kbc_diagnostics_noalloc(int nx, int ny, int variant, double beta,
     double* scratch = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_mu);
-        const unsigned long long ctx = current_context_id();
+        const unsigned long long ctx = current_context_id();  // 0: not cached
         if (!g_scratch_addr[dev] || ctx == 0 || g_scratch_ctx[dev] != ctx) {
             void* p = nullptr;
             if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
