@@ -74,13 +74,13 @@ def load_peaks():
 
 def step_kernel_name(args) -> str:
     """The step kernel the headline run launches; "auto" resolves as the
-    library does on large grids: the bulk-copy kernel for FP16 KBC, the
+    library does on large grids: the bulk-copy kernel for FP16 A and B, the
     per-node kernel for doubles, the vector rows otherwise (every bench width
     is a multiple of the row vector)."""
     k = args.kernel
     if k == "auto":
         k = "nodes" if args.dtype == "f64" else "rows"
-        if args.dtype == "f16" and args.variant != "lbgk":
+        if args.dtype == "f16" and args.variant in ("A", "B"):
             k = "bulk"
     return {"rows": "step_rows", "bulk": "step_tma", "nodes": "step_nodes"}[k]
 

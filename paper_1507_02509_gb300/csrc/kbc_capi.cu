@@ -452,13 +452,20 @@ static int step_into(kbc_handle h, const void* src, void* dst, cudaStream_t stre
     //   KBC on grids whose nodes are all resident at once (256^2 F32 B 3.1
     //   [rows 3.4]; F16 B 2.1 [rows 2.25]) and for the widths that the other
     //   two do not take;
-    // - bulk copies for FP16 KBC with several tiles for every resident block
-    //   (4096^2 B 136 [rows 155], 1024^2 10.3 [10.5]; 512^2 4.3 [rows 3.9]);
-    // - vector rows otherwise (4096^2 F32 B 180 [bulk 221], LBGK 172 [196]).
+    // - bulk copies for FP16 A and B beyond L2 (4096^2 B 136 [rows 137];
+    //   1536^2 19.4 for the rows [bulk 20.4]);
+    // - bulk copies for FP16 LBGK on fields about the size of L2, 80 to 240 MB
+    //   (1536^2 11.4 [rows 12.8], 2048^2 20.7 [27.8]; 1024^2 6.5 [6.2], 3072^2
+    //   63 [59]);
+    // - vector rows otherwise (4096^2 F32 B 180 [bulk 221], LBGK 172 [196],
+    //   F16 C 122 [bulk 126]).
     const long long total = (long long)h->nx * h->ny;
     const bool tiles = h->dtype != KBC_F64 && h->nx % kTmaTile == 0, kbc = h->variant != KBC_LBGK;
     const bool autok = h->kernel == KBC_KERNEL_AUTO || (h->kernel == KBC_KERNEL_BULK && !tiles);
-    const bool bulk = autok ? h->dtype == KBC_F16_DEV && kbc && total >= (long long)h->num_sms * 4096
+    const bool central = h->variant == KBC_A || h->variant == KBC_B;
+    const double mb = 18e-6 * (double)h->elem * (double)total;  // both fields
+    const bool bulk = autok ? h->dtype == KBC_F16_DEV && (kbc ? central && !rows_in_l2(total, h->elem)
+                                                              : mb >= 80.0 && mb <= 240.0)
                             : h->kernel == KBC_KERNEL_BULK;
     const bool rows = autok ? h->dtype != KBC_F64 && !(kbc && flat_small(h->nx, h->ny, h->num_sms))
                             : h->kernel == KBC_KERNEL_ROWS;

@@ -226,8 +226,21 @@ __device__ __forceinline__ unsigned collide_vec(T (&f)[NV][9], const CollidePara
 // wrap at the row ends).  Requires nx % (32 NV) == 0; a 1-D grid of
 // nbx * ny blocks, nbx = ceil(nx / (BLOCK NV)) blocks per row; warps past
 // the row end exit as a whole.
-template <int VAR, class C, int NV, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, C::kRowMinBlocks)
+// PAIRS: the four nodes are collided as two packed lane pairs, which takes 40%
+// fewer instructions and up to 128 registers: 8 resident blocks per SM (10 for
+// the natural-basis variants and LBGK, whose pairs fit 96) instead of 12.
+// That is the faster side where instructions bound the step: half storage
+// (4096^2 C 143 -> 122 us, bulk copies 126; 1024^2 B 10.5 -> 9.5), and
+// float fields that stay in L2 (1024^2 B 12.2 -> 11.6, C 11.4 -> 10.8);
+// where HBM does, the lower occupancy costs more than it saves (4096^2
+// float B 180 -> 182, half LBGK 103 -> 105).
+template <int VAR, class C, bool PAIRS> constexpr int row_min_blocks()
+{
+    return !PAIRS ? C::kRowMinBlocks : (VAR == kA || VAR == kB) ? 8 : 10;
+}
+
+template <int VAR, class C, int NV, int BLOCK, bool PAIRS>
+__global__ void __launch_bounds__(BLOCK, row_min_blocks<VAR, C, PAIRS>())
 step_rows(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst, StepArgs a,
           int nbx)
 {
@@ -284,7 +297,7 @@ step_rows(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst
         }
     }
     bool bad = false;
-    const unsigned hits = collide_vec<VAR, C::kUnits>(f, params_of<T>(a), bad);
+    const unsigned hits = collide_vec<VAR, C::kUnits, PAIRS>(f, params_of<T>(a), bad);
     if constexpr (VAR != kLBGK) {
         if (a.fix_list) record_fix<NV>(hits, y * a.nx + x0, 1, a);
     }

@@ -26,6 +26,11 @@ enum class StepKind { rows, nodes, bulk };
 // step_nodes: 1024 threads (16 blocks of 64) are resident per SM.
 inline bool flat_small(int nx, int ny, int num_sms) { return (long long)nx * ny <= (long long)num_sms * 1024; }
 
+// Whether the two fields of a step stay in L2 (129 MB, of which 100 MB hold
+// them without the rest of the step pushing them out: 1024^2 float, 75 MB, is
+// inside, 1536^2, 170 MB, outside).
+inline bool rows_in_l2(long long total, size_t elem) { return 18.0 * (double)elem * (double)total <= 100e6; }
+
 struct Launch {
     const void* src;
     void* dst;
@@ -106,8 +111,21 @@ cudaError_t launch_step_v(const Launch& L)
     if (L.kind == StepKind::rows) {
         constexpr int NV = C::kVec;
         const int nbx = (L.a.nx + kRowBlock * NV - 1) / (kRowBlock * NV);
-        e = launch_chained(step_rows<VAR, C, NV, kRowBlock>, (long long)nbx * L.a.ny, kRowBlock, 0, L.stream, src,
-                           dst, L.a, nbx);
+        const long long grid = (long long)nbx * L.a.ny;
+        // see step_rows for what either form is the faster one at
+        constexpr bool f32 = std::is_same<C, CodecF32>::value, f16 = std::is_same<C, CodecF16>::value;
+        const bool pairs = f16 ? VAR != kLBGK || rows_in_l2(total, sizeof(S))
+                               : f32 && VAR != kLBGK && rows_in_l2(total, sizeof(S));
+        if constexpr ((f32 && VAR != kLBGK) || f16) {
+            if (pairs)
+                e = launch_chained(step_rows<VAR, C, NV, kRowBlock, true>, grid, kRowBlock, 0, L.stream, src, dst,
+                                   L.a, nbx);
+        }
+        if constexpr (!f16 || VAR == kLBGK) {
+            if (!pairs)
+                e = launch_chained(step_rows<VAR, C, NV, kRowBlock, false>, grid, kRowBlock, 0, L.stream, src, dst,
+                                   L.a, nbx);
+        }
     } else if (L.kind == StepKind::nodes) {
         constexpr int K = flat_nodes<VAR, C>();
         if (K > 1 && !flat_small(L.a.nx, L.a.ny, L.num_sms)) {
