@@ -1296,17 +1296,32 @@ int kbc_adjoint(kbc_handle h, const double* rho0, const double* u0, int nsteps, 
     const int seglen = nsteps < K ? nsteps : K;
     const int nb = adj_blocks(n, h->num_sms);
     CallBuffers B(h);
-    // inputs on the device: rho0, u0 (and the target)
-    double* in = static_cast<double*>(B.get((size_t)(objective == 1 ? 5 : 3) * n * sizeof(double)));
-    double* gdev = static_cast<double*>(B.get((size_t)2 * n * sizeof(double)));
-    double* part = static_cast<double*>(B.get((size_t)(2 * nb + 8) * sizeof(double)));
-    void* work[2] = {B.get(field), B.get(field)};
-    void* lam[2] = {B.get(lamf), B.get(lamf)};
-    // one bit per node: single-precision reverse steps left to the double redo
+    // one allocation for everything but the checkpoints and states (each of
+    // ten took 10 us through the caller's allocator, half of what a step of
+    // a 512^2 grid takes): inputs rho0, u0 and the target; dJ/du0; sums; two
+    // fields, two lambdas; one bit per node for the single-precision reverse
+    // steps left to the double redo; a copy of a checkpoint
+    const bool even = K % 2 == 0 && h->graph_steps > 0;
     const size_t maskbytes = (size_t)((n + 31) / 32) * sizeof(unsigned);
-    unsigned* fixmask = static_cast<unsigned*>(B.get(maskbytes));
-    if (!in || !gdev || !part || !work[0] || !work[1] || !lam[0] || !lam[1] || !fixmask)
-        return fail(h, KBC_ERR_NOMEM, "adjoint buffers");
+    const size_t sizes[] = {(size_t)(objective == 1 ? 5 : 3) * n * sizeof(double), (size_t)2 * n * sizeof(double),
+                            (size_t)(2 * nb + 8) * sizeof(double), field, field, lamf, lamf, maskbytes,
+                            even && nsteps / K >= 2 ? field : 0};
+    void* piece[9];
+    size_t bytes = 0;
+    for (size_t b : sizes) bytes += (b + 255) & ~(size_t)255;
+    char* arena = static_cast<char*>(B.get(bytes));
+    if (!arena) return fail(h, KBC_ERR_NOMEM, "adjoint buffers");
+    for (int k = 0; k < 9; ++k) {
+        piece[k] = arena;
+        arena += (sizes[k] + 255) & ~(size_t)255;
+    }
+    double* in = static_cast<double*>(piece[0]);
+    double* gdev = static_cast<double*>(piece[1]);
+    double* part = static_cast<double*>(piece[2]);
+    void* work[2] = {piece[3], piece[4]};
+    void* lam[2] = {piece[5], piece[6]};
+    unsigned* fixmask = static_cast<unsigned*>(piece[7]);
+    void* ckwork = sizes[8] ? piece[8] : nullptr;
     // checkpoints and segment states in two slabs
     char* ckslab = nseg ? static_cast<char*>(B.get(field * (size_t)nseg)) : nullptr;
     char* segslab = seglen > 1 ? static_cast<char*>(B.get(field * (size_t)(seglen - 1))) : nullptr;
@@ -1322,9 +1337,7 @@ int kbc_adjoint(kbc_handle h, const double* rho0, const double* u0, int nsteps, 
     // float B, 100 steps in one segment: 3.8 -> 1.9 ms with both.
     AdjointGraphs G;
     const int last0 = nseg > 0 ? (nseg - 1) * K : 0;  // first step of the last segment
-    const bool even = K % 2 == 0 && h->graph_steps > 0;
     const bool fwd_graphs = even && nseg - 1 >= 2;    // every segment before the last is full
-    void* ckwork = (even && nsteps / K >= 2) ? B.get(field) : nullptr;
     const bool graphs = ckwork != nullptr;
     cudaError_t e = cudaMemcpyAsync(in, rho0, n * sizeof(double), cudaMemcpyDefault, h->stream);
     if (e == cudaSuccess)

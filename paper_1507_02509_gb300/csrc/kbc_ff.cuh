@@ -115,35 +115,38 @@ __device__ __forceinline__ void round_sure(float s, float t, float err, unsigned
     }
 }
 
-// Logarithms of 1 + x near 1 with eight FP64 instructions (the library's
-// log1p takes about thirty): the nearest multiple m of 1/128 from a table
-// {m, 1 / (1 + m), ln(1 + m)}, then ln(1 + r), r = (x - m) / (1 + m), as the
-// Taylor series to r^7, of which r^5 (1/5 - r/6 + r^2/7), 2^-28 of the whole,
-// needs no more than single precision.  For |x| < 1/2; the table is filled
-// by the kernel that uses it.
-struct LogTable {
+// (1 + x) ln(1 + x) near x = 0 with eight FP64 instructions (the library's
+// log1p alone takes about thirty): Taylor's series about the nearest multiple
+// m of 1/128, with r = (x - m) / (1 + m),
+//   (1 + m) ln(1 + m) + (1 + ln(1 + m)) (x - m) + (x - m) r (1/2 - r/6 + r^2/12 - ..),
+// of which r^2 (1/12 - r/20 + r^2/30), 2^-17 of the bracket, needs no more than
+// single precision.  For |x| < 1/2; the table is filled by the kernel that
+// uses it.
+struct EntropyTable {
     static constexpr int kHalf = 64;
-    double m[2 * kHalf + 1], c[2 * kHalf + 1], l[2 * kHalf + 1];
+    double m[2 * kHalf + 1], c[2 * kHalf + 1], f[2 * kHalf + 1], g[2 * kHalf + 1];
     __device__ __forceinline__ void fill()
     {
         for (int k = threadIdx.x; k <= 2 * kHalf; k += blockDim.x) {
             m[k] = (double)(k - kHalf) * (0.5 / kHalf);
             c[k] = 1.0 / (1.0 + m[k]);
-            l[k] = log1p(m[k]);
+            const double l = log1p(m[k]);
+            f[k] = (1.0 + m[k]) * l;
+            g[k] = 1.0 + l;
         }
     }
-    // x in double and rounded to float (to about 2^-20 of itself)
-    __device__ __forceinline__ double log1p_near(double x, float xf) const
+    // x in double and as a float (to about 2^-20 of itself)
+    __device__ __forceinline__ double entropy_near(double x, float xf) const
     {
         const int k = __float2int_rn(xf * (2.0f * kHalf)) + kHalf;
-        const double r = (x - m[k]) * c[k];
+        const double d = x - m[k];
+        const double r = d * c[k];
         const float mf = (float)(k - kHalf) * (0.5f / kHalf);
         const float rf = (xf - mf) * __fdividef(1.0f, 1.0f + mf);
-        const float g = __fmaf_rn(rf, __fmaf_rn(rf, 1.0f / 7.0f, -1.0f / 6.0f), 0.2f);
-        double h = __fma_rn(r, widen_normal(g), -0.25);
-        h = __fma_rn(r, h, 1.0 / 3.0);
-        h = __fma_rn(r, h, -0.5);
-        return l[k] + __fma_rn(r * r, h, r);
+        const float s = __fmaf_rn(rf, __fmaf_rn(rf, 1.0f / 30.0f, -1.0f / 20.0f), 1.0f / 12.0f);
+        double h = __fma_rn(r, widen_normal(s), -1.0 / 6.0);
+        h = __fma_rn(r, h, 0.5);
+        return __fma_rn(g[k], d, __fma_rn(d * r, h, f[k]));
     }
 };
 
