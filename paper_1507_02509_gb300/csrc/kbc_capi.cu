@@ -274,6 +274,7 @@ struct kbc_ctx {
     int cur = 0;          // buffer holding the current state
     int* fix = nullptr;   // [0..1] counters, [64..] list of node indices
     int fix_slot = 0;
+    int sweep = 0;        // direction of the next step (results do not depend on it)
     int* flag_dev = nullptr;
     int* flag_host = nullptr;  // pinned
     double* diag_part = nullptr;
@@ -376,6 +377,7 @@ StepArgs args_of(const kbc_ctx* h)
     a.fix_list = h->fix ? h->fix + 64 : nullptr;
     a.fix_slot = h->fix_slot;
     a.flag = h->flag_dev;
+    a.rev = 0;
     a.ywrap = h->slab ? 0 : 1;
     return a;
 }
@@ -481,6 +483,8 @@ static int step_into(kbc_handle h, const void* src, void* dst, cudaStream_t stre
     L.src = src;
     L.dst = dst;
     L.a = args_of(h);
+    L.a.rev = h->sweep && !rows_in_l2(total, h->elem);
+    h->sweep ^= 1;
     if (!guard_on) L.a.fix_list = nullptr;
     cudaError_t e = by_codec(h->dtype, [&](auto c) {
         using C = decltype(c);
@@ -1655,7 +1659,10 @@ int kbc_slabs_step(int parts, const kbc_handle* slabs, int nsteps)
     for (int s = 0; s < nsteps; ++s) {
         e = group_halos(parts, hs.data());
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "slab halos");
-        for (kbc_handle h : hs) {
+        const int back = hs[0]->sweep;
+        for (int k = 0; k < parts; ++k) {
+            kbc_handle h = hs[back ? parts - 1 - k : k];  // one sweep over the whole grid
+            h->sweep = back;
             h->ghosts_full = 0;
             const int rc = step_into(h, h->buf[h->cur], h->buf[h->cur ^ 1]);
             if (rc) return fail(nullptr, rc, h->err);

@@ -284,7 +284,7 @@ step_guard(const float* __restrict__ src, float* __restrict__ dst, StepArgs a, G
                     for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = out[i];
                 }
             }
-            // every lane has read its entry before entries of this round are overwritten
+            // every lane has read its entry before entries it may overwrite
             const unsigned vote = __ballot_sync(0xffffffffu, open);
             if (open) a.fix_list[w0 + kept + __popc(vote & ((1u << lane) - 1u))] = n;
             kept += __popc(vote);

@@ -180,6 +180,8 @@ step_tma(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst,
     const int tiles = tiles_per_row * a.ny;
     const int first = blockIdx.x, stride = gridDim.x;
     const int my_tiles = first < tiles ? (tiles - 1 - first) / stride + 1 : 0;
+    // the tile of this block's turn k, from the field's end where a.rev (see sweep_block)
+    auto tile_of = [&](int k) { return a.rev ? tiles - 1 - (first + k * stride) : first + k * stride; };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -209,7 +211,7 @@ step_tma(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst,
                 }
                 if (abort_flag) break;
                 tma_issue<S, TX>(src, stage_buf + (size_t)s * 9 * ROW, &full[s],
-                                 first + k * stride, tiles_per_row, a);
+                                 tile_of(k), tiles_per_row, a);
             }
         }
         return;
@@ -227,7 +229,7 @@ step_tma(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst,
             abort_flag = 1;
             break;
         }
-        const int t = first + k * stride;
+        const int t = tile_of(k);
         const int y = t / tiles_per_row;
         const int x0 = (t - y * tiles_per_row) * TX;
         const S* buf = stage_buf + (size_t)s * 9 * ROW;
