@@ -644,8 +644,8 @@ def next_rows_extras(args, rho, ux, uy, beta, peak, stream):
     grp.close()
     res["slabs_4_on_one_gpu"] = {"mlups": round(nodes / t / 1e6, 1),
                                  "frac": round(72.0 * nodes / t / 1e9 / peak, 4),
-                                 "what": "the grid as four y-slabs with a halo exchange (two "
-                                         "device copies per slab) before every step"}
+                                 "what": "the grid as four y-slabs with a halo exchange (one "
+                                         "kernel for all slabs) before every step"}
     return res
 
 

@@ -56,8 +56,8 @@ __device__ __forceinline__ Ld fmaL(Ld a, Ld b, Ld c) { return Ld(__fma_rn(a.v, b
 __device__ __forceinline__ Ld rcp_fast(Ld x) { return Ld(rcp_pos(x.v)); }
 // a / b as a times the reciprocal of b (in the double collision it forms
 // gamma*'s ratio <ds|dh> / <dh|dh>).  rcp_pos for this and for 1 / rho instead
-// of the correctly rounded reciprocal: 201 -> 189 FP64 instructions a node of
-// the step, whose FP64 pipe is the bound (1024^2 B 384 -> 362 us).
+// of the correctly rounded reciprocal: 201 -> 196 FP64 instructions a node of
+// the step, whose FP64 pipe is the bound (1024^2 B 384 -> 373 us).
 __device__ __forceinline__ Ld ratio(Ld a, Ld b) { return Ld(__dmul_rn(a.v, rcp_pos(b.v))); }
 __device__ __forceinline__ unsigned gt_mask(Ld a, Ld b) { return a.v > b.v ? 1u : 0u; }
 __device__ __forceinline__ unsigned finite_mask(Ld a) { return isfinite(a.v) ? 1u : 0u; }
