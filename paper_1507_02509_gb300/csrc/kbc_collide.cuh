@@ -70,15 +70,9 @@ __host__ inline CollideParams<T> make_params(double beta, int fixed, double gamm
     return p;
 }
 
-// Fast reciprocal / quotient: float uses the approximate hardware path
-// (__fdividef, 2 ulp); double the IEEE operations.
-template <typename T> __device__ __forceinline__ T rcp_fast(T x);
-template <> __device__ __forceinline__ float rcp_fast<float>(float x) { return __fdividef(1.0f, x); }
-template <> __device__ __forceinline__ double rcp_fast<double>(double x) { return 1.0 / x; }
-
-template <typename T> __device__ __forceinline__ T ratio(T a, T b);
-template <> __device__ __forceinline__ float ratio<float>(float a, float b) { return __fdividef(a, b); }
-template <> __device__ __forceinline__ double ratio<double>(double a, double b) { return a / b; }
+// The lanes' reciprocal for a plain float: the approximate hardware path
+// (__fdividef, 2 ulp).
+__device__ __forceinline__ float rcp_fast(float x) { return __fdividef(1.0f, x); }
 
 // P_i = 3 xi + 4.5 xi^2 - 1.5 u^2 with xi = v_i . u, so that
 // f^eq_i = W_i rho (1 + P_i) (Eq. Eq).  Opposite velocities share one xi:

@@ -145,7 +145,7 @@ cudaError_t launch_step_v(const Launch& L)
                 gp.nb = (float)(-L.a.pd.one_m_2beta);
                 gp.settle = (double)L.a.pf.guard <= kGuardSettle;
                 e = launch_chained(step_guard<VAR>, L.num_sms, kGuardBlock, 0, L.stream, src, dst, L.a, gp);
-            } else {
+            } else if constexpr (std::is_same<C, CodecF16>::value) {
                 e = launch_chained(step_fixup<VAR, C>, L.num_sms * 2, kNodeBlock, 0, L.stream, src, dst, L.a);
             }
         }
