@@ -15,6 +15,7 @@
 
 #include "../../include/kbc.h"
 #include "kbc_launch.cuh"
+#include "kbc_pools.cuh"
 #include "kbc_slab.cuh"
 #include "kbc_spectrum.cuh"
 
@@ -116,138 +117,76 @@ int kbc::handle_free_error(int code, const char* msg)
     return code;
 }
 
+// A driver function by its name, nullptr when the driver has none.
+template <class F>
+static F driver_entry(const char* name, unsigned version)
+{
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPointByVersion(name, &fn, version, cudaEnableDefault, &q) == cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    cudaGetLastError();
+    return ok ? reinterpret_cast<F>(fn) : nullptr;
+}
+
 unsigned long long kbc::current_context_id()
 {
-    static const PFN_cuCtxGetId_v12000 get_id = [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const bool ok = cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &q) ==
-                            cudaSuccess &&
-                        q == cudaDriverEntryPointSuccess;
-        cudaGetLastError();
-        return ok ? reinterpret_cast<PFN_cuCtxGetId_v12000>(fn) : nullptr;
-    }();
+    static const auto get_id = driver_entry<PFN_cuCtxGetId_v12000>("cuCtxGetId", 12000);
     unsigned long long id = 0;
     if (!get_id || get_id(nullptr, &id) != CUDA_SUCCESS) return 0;
     return id;
 }
 
-// Host resources kept between objects and calls, because making them costs
-// more than a small problem computes.  Both are bounded, handed out to one
-// owner at a time under a lock, and belong to the context they were made in.
-//
-// Pinned status words of the handles: 256 slots of one page (the first
-// pinned allocation of a process without one takes 230 us; creating and
-// destroying a handle 398 -> 165 us).
 namespace {
 
-struct FlagPool {
-    static constexpr int kSlots = 256, kInts = 4;
-    std::mutex mu;
-    int* page = nullptr;
-    unsigned long long ctx = 0;
-    bool used[kSlots] = {};
+// whether the current context is its device's primary one
+bool in_primary_context(int device)
+{
+    static const auto current = driver_entry<PFN_cuCtxGetCurrent_v4000>("cuCtxGetCurrent", 4000);
+    static const auto retain = driver_entry<PFN_cuDevicePrimaryCtxRetain_v7000>("cuDevicePrimaryCtxRetain", 7000);
+    static const auto release = driver_entry<PFN_cuDevicePrimaryCtxRelease_v11000>("cuDevicePrimaryCtxRelease", 11000);
+    CUcontext cur = nullptr, primary = nullptr;
+    if (!current || !retain || !release || current(&cur) != CUDA_SUCCESS || !cur) return false;
+    if (retain(&primary, device) != CUDA_SUCCESS) return false;
+    release(device);
+    return cur == primary;
+}
 
-    int* get()
+struct PoolRuntime {
+    using Plan = cufftHandle;
+    static Context context()
     {
-        std::lock_guard<std::mutex> lk(mu);
-        const unsigned long long id = current_context_id();
-        if (id != 0 && (!page || ctx != id)) {  // another context's page went with it
-            page = nullptr;
-            if (cudaHostAlloc((void**)&page, kSlots * kInts * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
-                cudaGetLastError();
-                page = nullptr;
-            }
-            ctx = id;
-            for (bool& u : used) u = false;
+        Context c;
+        if (cudaGetDevice(&c.device) != cudaSuccess) {
+            cudaGetLastError();
+            return Context();
         }
-        for (int k = 0; page && id == ctx && k < kSlots; ++k)
-            if (!used[k]) {
-                used[k] = true;
-                return page + k * kInts;
-            }
-        int* own = nullptr;
-        if (cudaHostAlloc((void**)&own, kInts * sizeof(int), cudaHostAllocDefault) != cudaSuccess) return nullptr;
-        return own;
+        // the number of a runtime device is the driver's
+        if (in_primary_context(c.device)) c.id = current_context_id();
+        return c;
     }
-    // the caller has waited for every copy into it
-    void put(int* p)
+    static int* host_alloc(size_t bytes, bool portable)
     {
-        if (!p) return;
-        std::lock_guard<std::mutex> lk(mu);
-        if (page && p >= page && p < page + kSlots * kInts) used[(p - page) / kInts] = false;
-        else cudaFreeHost(p);
+        int* p = nullptr;
+        const unsigned flags = portable ? cudaHostAllocPortable : cudaHostAllocDefault;
+        if (cudaHostAlloc((void**)&p, bytes, flags) == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
     }
+    static void host_free(int* p) { cudaFreeHost(p); }
+    static bool plan_create(int n, Plan* plan, size_t* work)
+    {
+        if (cufftCreate(plan) != CUFFT_SUCCESS) return false;
+        if (cufftSetAutoAllocation(*plan, 0) == CUFFT_SUCCESS &&
+            cufftMakePlan2d(*plan, n, n, CUFFT_Z2Z, work) == CUFFT_SUCCESS)
+            return true;
+        cufftDestroy(*plan);
+        return false;
+    }
+    static void plan_destroy(Plan plan) { cufftDestroy(plan); }
 };
-FlagPool g_flags;
-
-// cuFFT plans of kbc_spectrum by size (making one takes 0.3 to 0.5 ms, more
-// than the transform of a 1024^2 field); the work area is the call's own.
-struct PlanPool {
-    static constexpr int kPlans = 8;
-    struct Entry {
-        cufftHandle plan = 0;
-        size_t work = 0;
-        int n = 0, device = -1;
-        unsigned long long ctx = 0, age = 0;
-        bool held = false;
-    };
-    std::mutex mu;
-    Entry e[kPlans];
-    unsigned long long clock = 0;
-
-    // a plan that nobody else uses until put(); false when cuFFT fails
-    bool get(int n, int device, Entry* out)
-    {
-        const unsigned long long id = current_context_id();
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            for (Entry& x : e)
-                if (x.held && id != 0 && x.n == n && x.device == device && x.ctx == id) {
-                    *out = x;
-                    x = Entry();
-                    return true;
-                }
-        }
-        Entry x;
-        if (cufftCreate(&x.plan) != CUFFT_SUCCESS) return false;
-        if (cufftSetAutoAllocation(x.plan, 0) != CUFFT_SUCCESS ||
-            cufftMakePlan2d(x.plan, n, n, CUFFT_Z2Z, &x.work) != CUFFT_SUCCESS) {
-            cufftDestroy(x.plan);
-            return false;
-        }
-        x.n = n;
-        x.device = device;
-        x.ctx = id;
-        *out = x;
-        return true;
-    }
-    // the caller has waited for the plan's work
-    void put(Entry x)
-    {
-        Entry old;
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            Entry* to = &e[0];
-            for (Entry& y : e) {
-                if (!y.held) {
-                    to = &y;
-                    break;
-                }
-                if (y.age < to->age) to = &y;
-            }
-            old = *to;
-            x.held = x.ctx != 0;
-            x.age = ++clock;
-            if (x.held) *to = x;
-            else old = x, old.held = true;
-        }
-        // the least recently used one makes room; one of a context that is
-        // gone went with it
-        if (old.held && (old.ctx == 0 || old.ctx == current_context_id())) cufftDestroy(old.plan);
-    }
-};
-PlanPool g_plans;
+FlagPool<PoolRuntime> g_flags;
+PlanPool<PoolRuntime> g_plans;
 
 }  // namespace
 
@@ -276,6 +215,7 @@ struct kbc_ctx {
     int fix_slot = 0;
     int sweep = 0;        // direction of the next step (results do not depend on it)
     int* flag_dev = nullptr;
+    FlagWords flag_words;      // what flag_host points into
     int* flag_host = nullptr;  // pinned
     double* diag_part = nullptr;
     int diag_nblocks = 0;
@@ -818,9 +758,9 @@ static int create_common(int nx, int ny, int variant, double beta, int dtype, bo
         kbc_destroy(h);
         return fail(nullptr, KBC_ERR_NOMEM, "device allocation failed");
     }
-    h->flag_host = g_flags.get();
+    h->flag_words = g_flags.get();
+    h->flag_host = h->flag_words.p;
     if (!h->flag_host) {
-        cudaGetLastError();
         kbc_destroy(h);
         return fail(nullptr, KBC_ERR_CUDA, "pinned allocation failed");
     }
@@ -863,7 +803,7 @@ int kbc_destroy(kbc_handle h)
     dev_free(h, h->diag_part);
     dev_free(h, h->diag_out);
     dev_free(h, h->stage);
-    g_flags.put(h->flag_host);
+    g_flags.put(h->flag_words);
     drop_graphs(h);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
@@ -1701,7 +1641,7 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
         cudaStream_t s;
         void* p[4] = {nullptr, nullptr, nullptr, nullptr};
         int k = 0;
-        PlanPool::Entry fft;
+        PlanPool<PoolRuntime>::Entry fft;
         bool planned = false;
         void* get(size_t bytes)
         {
@@ -1742,7 +1682,7 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (!g_plans.get(n, dev, &sc.fft)) return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT plan");
+    if (!g_plans.get(n, &sc.fft)) return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT plan");
     sc.planned = true;
     void* work = sc.get(sc.fft.work);
     if (!work) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: cuFFT work area allocation failed");
