@@ -205,9 +205,12 @@ int kbc_set_kernel(kbc_handle h, int kernel);
 
 /* kbc_step replays a CUDA graph of `steps` consecutive steps (captured once
  * per handle configuration on a private stream, then launched on the bound
- * stream) for as many whole graphs as nsteps holds, and launches the rest
- * one by one; this removes the per-launch overhead that dominates small
- * grids.  Graphs give the same bits as individual launches.  steps must be
+ * stream) for as many whole graphs as nsteps holds.  The rest is launched step
+ * by step; when two calls before ended with the same number of steps, its even
+ * part, from four steps on, is replayed as a graph of its own (kept for the
+ * last four such numbers).  This removes the per-launch overhead that
+ * dominates small grids; making and dropping graphs does not wait for the
+ * stream.  Graphs give the same bits as individual launches.  steps must be
  * even (the two population buffers return to their roles after an even
  * count); 0 disables graphs.  Default 32.  Not used while the bound stream
  * is itself being captured. */

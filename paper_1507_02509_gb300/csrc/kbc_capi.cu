@@ -195,6 +195,18 @@ PlanPool<PoolRuntime> g_plans;
 constexpr int kPipeChunks = 32;
 constexpr size_t kPipeMinBytes = (size_t)64 << 20;
 
+// Graphs of one number of steps in one configuration, by (cur, fix_slot)
+// parity; seen: the steps that were launched singly.
+struct ShortRun {
+    int len = 0;
+    unsigned config = 0;
+    int seen[4] = {0, 0, 0, 0};
+    unsigned version[4] = {0, 0, 0, 0};
+    cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
+    unsigned long long age = 0;
+};
+constexpr int kShortRuns = 4;
+
 struct kbc_ctx {
     int nx = 0, ny = 0, variant = 0, dtype = 0, device = 0, num_sms = 1;
     double beta = 1.0;
@@ -230,11 +242,10 @@ struct kbc_ctx {
     unsigned config_version = 1;
     unsigned graph_version[4] = {0, 0, 0, 0};
     cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
-    // the same for the even number of steps below graph_steps that the last
-    // two calls ended with (short_len; captured when it is seen again)
-    int short_len = 0;
-    unsigned short_version[4] = {0, 0, 0, 0};
-    cudaGraphExec_t short_graph[4] = {nullptr, nullptr, nullptr, nullptr};
+    // the same for even numbers of steps below graph_steps, which calls end
+    // with: the few lengths asked for last
+    ShortRun short_run[kShortRuns];
+    unsigned long long short_clock = 0;
     cudaStream_t capture_stream = nullptr;
     // host <-> device pipelines: copies of one row chunk overlap the kernel
     // of the neighbouring chunk on this second stream, ordered by events
@@ -466,16 +477,13 @@ static cudaGraphExec_t capture_work(kbc_handle h, F&& issue)
     return exec;
 }
 
-static void drop_short_graphs(kbc_handle h)
+// A replay may still run: the runtime keeps what it needs of a destroyed graph
+// until it has completed, so that nothing here waits.
+static void drop_short(ShortRun& r)
 {
-    bool any = false;
-    for (cudaGraphExec_t g : h->short_graph) any |= g != nullptr;
-    if (any) cudaStreamSynchronize(h->stream);  // the last replay may still run
-    for (int k = 0; k < 4; ++k) {
-        if (h->short_graph[k]) cudaGraphExecDestroy(h->short_graph[k]);
-        h->short_graph[k] = nullptr;
-        h->short_version[k] = 0;
-    }
+    for (cudaGraphExec_t g : r.graph)
+        if (g) cudaGraphExecDestroy(g);
+    r = ShortRun();
 }
 
 static void drop_graphs(kbc_handle h)
@@ -485,8 +493,7 @@ static void drop_graphs(kbc_handle h)
         h->graph[k] = nullptr;
         h->graph_version[k] = 0;
     }
-    drop_short_graphs(h);
-    h->short_len = 0;
+    for (ShortRun& r : h->short_run) drop_short(r);
 }
 
 // The instantiated graph of `steps` (even) steps starting from the current
@@ -513,6 +520,27 @@ static cudaGraphExec_t step_graph(kbc_handle h, int steps, cudaGraphExec_t* slot
         version[key] = h->config_version;
     }
     return exec;
+}
+
+// The entry of calls that end with `steps` single steps: a free one, or the
+// least recently used one, when there is none.
+static ShortRun& short_run(kbc_handle h, int steps)
+{
+    ShortRun* to = nullptr;
+    for (ShortRun& r : h->short_run) {
+        if (r.len == steps) {
+            to = &r;
+            break;
+        }
+        if (!to || r.age < to->age) to = &r;  // a free one has age 0
+    }
+    if (to->len != steps || to->config != h->config_version) {
+        drop_short(*to);
+        to->len = steps;
+        to->config = h->config_version;
+    }
+    to->age = ++h->short_clock;
+    return *to;
 }
 
 // Graphs of one kbc_adjoint call (its buffers are the call's own).
@@ -969,22 +997,23 @@ int kbc_step(kbc_handle h, int nsteps)
         }
     }
     // The rest below graph_steps: programs that take a few steps between looks
-    // at the field ask for the same number again and again, and launching
+    // at the field ask for the same few numbers again and again, and launching
     // them one by one costs more than small grids compute (128^2, float C, ten
-    // steps: 20 launches, 56 us, against 25 us for the replay).  One call of a
-    // length launches directly, so that it does not pay for a capture.
+    // steps: 63 us, the replay 45).  A capture costs what the replays of a few
+    // calls save (another 60 us there), so the first two calls of a length
+    // launch directly, and the first 20 steps: a program of few calls does not
+    // pay for it, one that alternates between a few lengths pays once for each
+    // (10, 10 and 7 steps 257 us with single launches, 111 now).
     const int rest = (nsteps - done) & ~1;
     if (h->graph_steps > 0 && rest >= 4 && !capturing) {
-        if (rest == h->short_len) {
-            cudaGraphExec_t g = step_graph(h, rest, h->short_graph, h->short_version);
-            if (g) {
-                cudaError_t e = cudaGraphLaunch(g, h->stream);
-                if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
-                done += rest;
-            }
-        } else {
-            drop_short_graphs(h);
-            h->short_len = rest;
+        ShortRun& r = short_run(h, rest);
+        int& seen = r.seen[h->cur | (h->fix_slot << 1)];
+        if (seen < 2 * rest || seen < 20) {
+            seen += rest;
+        } else if (cudaGraphExec_t g = step_graph(h, rest, r.graph, r.version)) {
+            cudaError_t e = cudaGraphLaunch(g, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
+            done += rest;
         }
     }
     for (int s = done; s < nsteps; ++s) {

@@ -1,0 +1,67 @@
+"""Short runs of several lengths: replays of the lengths asked for last, whose
+exchange does not wait for the stream."""
+import pytest
+
+from gpu_helpers import random_field, representable
+
+pytestmark = pytest.mark.gpu
+
+NX, NY, BETA = 96, 33, 0.97
+
+
+def pair(dtype, variant):
+    from paper_1507_02509_gb300 import Lattice
+
+    g = representable(random_field(NX, NY, 6, amp=1e-3), dtype)
+    a, b = (Lattice(NX, NY, variant=variant, beta=BETA, dtype=dtype) for _ in range(2))
+    b.set_graph_steps(0)
+    for lat in (a, b):
+        lat.set_populations(g)
+    return a, b
+
+
+def busy(seconds=0.25):
+    import torch
+
+    torch.cuda._sleep(int(seconds * 2.07e9))  # at most: the clock's highest rate
+
+
+@pytest.mark.parametrize("dtype,variant", [("f64", "B"), ("f32", "A"), ("f16", "D")])
+def test_alternating_and_evicted_lengths_give_the_bits_of_single_launches(dtype, variant):
+    import torch
+
+    a, b = pair(dtype, variant)
+    # a pattern of two lengths with a change of parity, then more lengths than are kept
+    lengths = [10, 10, 7] * 6 + [n for n in (4, 6, 8, 12, 14, 16) for _ in range(7)] + [10, 7, 44, 42] * 4
+    for n in lengths:
+        a.step(n)
+        b.step(n)
+    assert torch.equal(a.populations(), b.populations())
+    a.close()
+    b.close()
+
+
+def test_a_changed_length_does_not_wait_for_the_stream():
+    import torch
+
+    a, b = pair("f32", "B")
+    lengths = [n for n in (4, 6, 8, 10, 12, 14) for _ in range(7)]
+    for n in lengths:  # graphs of every kept length
+        a.step(n)
+        b.step(n)
+    torch.cuda.synchronize()
+    busy()
+    a.step(14)  # replays of what is dropped below wait behind the sleep
+    for n in lengths:
+        a.step(n)
+    a.set_graph_steps(16)
+    a.step(6)
+    waited = torch.cuda.current_stream().query()
+    b.step(14)
+    for n in lengths:
+        b.step(n)
+    b.step(6)
+    assert not waited
+    assert torch.equal(a.populations(), b.populations())
+    a.close()
+    b.close()
