@@ -446,6 +446,17 @@ static int step_into(kbc_handle h, const void* src, void* dst, cudaStream_t stre
     return KBC_OK;
 }
 
+// While it lives, this thread's calls that make or destroy graphs are none of
+// the business of captures under way elsewhere: without it they fail, and
+// spoil the other capture, while any thread of the process captures in the
+// global mode (the default of PyTorch's graphs).
+struct GraphCalls {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    GraphCalls() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~GraphCalls() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    GraphCalls(const GraphCalls&) = delete;
+};
+
 // Instantiated graph of the work `issue(stream)` enqueues on the private
 // capture stream (returns false on a failed launch); nullptr when capture or
 // instantiation fails, with the handle's guard parity restored, so that the
@@ -453,6 +464,7 @@ static int step_into(kbc_handle h, const void* src, void* dst, cudaStream_t stre
 template <class F>
 static cudaGraphExec_t capture_work(kbc_handle h, F&& issue)
 {
+    const GraphCalls relaxed;
     if (!h->capture_stream &&
         cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
@@ -481,6 +493,7 @@ static cudaGraphExec_t capture_work(kbc_handle h, F&& issue)
 // until it has completed, so that nothing here waits.
 static void drop_short(ShortRun& r)
 {
+    const GraphCalls relaxed;
     for (cudaGraphExec_t g : r.graph)
         if (g) cudaGraphExecDestroy(g);
     r = ShortRun();
@@ -488,6 +501,7 @@ static void drop_short(ShortRun& r)
 
 static void drop_graphs(kbc_handle h)
 {
+    const GraphCalls relaxed;
     for (int k = 0; k < 4; ++k) {
         if (h->graph[k]) cudaGraphExecDestroy(h->graph[k]);
         h->graph[k] = nullptr;
@@ -503,6 +517,7 @@ static cudaGraphExec_t step_graph(kbc_handle h, int steps, cudaGraphExec_t* slot
 {
     const int key = h->cur | (h->fix_slot << 1);
     if (slot[key] && version[key] == h->config_version) return slot[key];
+    const GraphCalls relaxed;
     if (slot[key]) {
         cudaGraphExecDestroy(slot[key]);
         slot[key] = nullptr;
@@ -551,6 +566,7 @@ struct AdjointGraphs {
     cudaGraphExec_t rev[2] = {nullptr, nullptr}; // reverse segment, by lambda parity
     ~AdjointGraphs()
     {
+        const GraphCalls relaxed;
         for (cudaGraphExec_t g : {fwd, rec[0], rec[1], rev[0], rev[1]})
             if (g) cudaGraphExecDestroy(g);
     }

@@ -1,5 +1,5 @@
 """Short runs of several lengths: replays of the lengths asked for last, whose
-exchange does not wait for the stream."""
+exchange neither waits for the stream nor disturbs a capture."""
 import pytest
 
 from gpu_helpers import random_field, representable
@@ -65,3 +65,74 @@ def test_a_changed_length_does_not_wait_for_the_stream():
     assert torch.equal(a.populations(), b.populations())
     a.close()
     b.close()
+
+
+def test_graphs_dropped_while_the_stream_is_captured():
+    import torch
+
+    a, b = pair("f32", "C")
+    for _ in range(4):
+        a.step(10)
+        b.step(10)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        a.set_graph_steps(64)
+        a.step(4)
+    graph.replay()
+    graph.replay()
+    b.step(8)
+    assert torch.equal(a.populations(), b.populations())
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("thread", [False, True])
+def test_short_runs_beside_a_capture(thread):
+    """A handle on a stream of its own takes, repeats and exchanges short runs
+    while another handle's steps are captured in the global mode."""
+    import threading
+
+    import torch
+
+    from paper_1507_02509_gb300 import Lattice
+
+    a, b = pair("f32", "B")
+    s = torch.cuda.Stream()
+    g = a.populations()
+    lat = Lattice(NX, NY, variant="B", beta=BETA, dtype="f32", stream=s)
+    lat.set_populations(g)
+    torch.cuda.synchronize()
+    lengths = [n for n in (10, 4, 6, 8, 12) for _ in range(7)]
+    failed = []
+
+    def run():
+        try:
+            for n in lengths:
+                lat.step(n)
+            lat.set_graph_steps(16)
+            lat.step(40)
+        except Exception as e:
+            failed.append(e)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        a.step(4)
+        if thread:
+            t = threading.Thread(target=run)
+            t.start()
+            t.join()
+        else:
+            run()
+        a.step(4)
+    assert not failed, failed
+    graph.replay()
+    b.step(8)
+    assert torch.equal(a.populations(), b.populations())
+    b.set_populations(g)
+    for n in lengths + [40]:
+        b.step(n)
+    s.synchronize()
+    assert torch.equal(lat.populations(), b.populations())
+    for x in (a, b, lat):
+        x.close()
