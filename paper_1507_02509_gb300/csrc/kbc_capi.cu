@@ -252,7 +252,10 @@ struct kbc_ctx {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t pipe_ev[kPipeChunks + 2] = {};
     cudaStream_t stream = nullptr;
-    bool restreamed = false;  // another stream was bound while there was work
+    // work of the handle may be on streams other than the bound one: another
+    // was bound while there was work, or steps were captured by the caller,
+    // whose replays go where the caller launches them
+    bool elsewhere = false;
     Allocator al;
     std::string err;
 };
@@ -838,7 +841,7 @@ int kbc_destroy(kbc_handle h)
     if (!h) return KBC_ERR_ARG;
     cudaSetDevice(h->device);
     // every stream that may still write the handle's status words
-    if (h->restreamed) cudaDeviceSynchronize();
+    if (h->elsewhere) cudaDeviceSynchronize();
     else cudaStreamSynchronize(h->stream);
     dev_free(h, h->alloc[0]);
     dev_free(h, h->alloc[1]);
@@ -861,7 +864,7 @@ int kbc_destroy(kbc_handle h)
 int kbc_set_stream(kbc_handle h, void* stream)
 {
     if (!h) return KBC_ERR_ARG;
-    if (h->initialized && h->stream != static_cast<cudaStream_t>(stream)) h->restreamed = true;
+    if (h->initialized && h->stream != static_cast<cudaStream_t>(stream)) h->elsewhere = true;
     h->stream = static_cast<cudaStream_t>(stream);
     return KBC_OK;
 }
@@ -986,6 +989,14 @@ int kbc_get_populations(kbc_handle h, double* f)
     });
 }
 
+static bool is_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool yes = cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return yes;
+}
+
 int kbc_step(kbc_handle h, int nsteps)
 {
     int rc = check_h(h);
@@ -999,10 +1010,8 @@ int kbc_step(kbc_handle h, int nsteps)
     if (nsteps == 0) return KBC_OK;
     h->ghosts_full = 0;
     int done = 0;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const bool capturing = cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess ||
-                           cs != cudaStreamCaptureStatusNone;
-    cudaGetLastError();
+    const bool capturing = is_capturing(h->stream);
+    h->elsewhere |= capturing;
     if (h->graph_steps > 0 && nsteps >= h->graph_steps && !capturing) {
         cudaGraphExec_t g = step_graph(h, h->graph_steps, h->graph, h->graph_version);
         if (g) {
@@ -1641,6 +1650,8 @@ int kbc_slabs_step(int parts, const kbc_handle* slabs, int nsteps)
     }
     cudaError_t e = cudaSetDevice(hs[0]->device);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaSetDevice");
+    const bool capturing = is_capturing(hs[0]->stream);
+    for (kbc_handle h : hs) h->elsewhere |= capturing;
     for (int s = 0; s < nsteps; ++s) {
         e = group_halos(parts, hs.data());
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "slab halos");

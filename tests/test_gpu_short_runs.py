@@ -136,3 +136,28 @@ def test_short_runs_beside_a_capture(thread):
     assert torch.equal(lat.populations(), b.populations())
     for x in (a, b, lat):
         x.close()
+
+
+@pytest.mark.parametrize("slabs", [False, True])
+def test_destroying_a_handle_waits_for_replays_of_its_captured_steps(slabs):
+    """A replay copies into the handle's status word, on whatever stream it is
+    launched: the word is not given to another handle before it has ended."""
+    import torch
+
+    from paper_1507_02509_gb300 import Lattice
+    from paper_1507_02509_gb300.slabs import SlabGroup
+
+    s, t = torch.cuda.Stream(), torch.cuda.Stream()
+    kw = dict(variant="B", beta=BETA, dtype="f32", stream=s)
+    x = SlabGroup(NX, NY, 2, **kw) if slabs else Lattice(NX, NY, **kw)
+    with torch.cuda.stream(s):
+        x.set_populations(torch.as_tensor(random_field(NX, NY, 6, amp=1e-3)).cuda())
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        x.step(2)
+    with torch.cuda.stream(t):
+        busy()
+        graph.replay()
+    x.close()
+    assert t.query()
