@@ -137,9 +137,13 @@ class SlabGroup:
     def step(self, n: int = 1):
         """n steps, halos first each time, as one call of the library
         (kbc_slabs_step): one halo kernel for all slabs and one launch per
-        slab and step, instead of four copies and three calls per slab."""
+        slab and step, instead of four copies and three calls per slab.
+        No steps (n < 1) ask nothing of the slabs."""
         from . import capi
 
+        n = int(n)
+        if n < 1:
+            return self
         for s in self.slabs:
             s._bind_stream()
         capi.kbc_slabs_step([s.h for s in self.slabs], n)
