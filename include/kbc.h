@@ -329,9 +329,10 @@ int kbc_diagnostics_ext(kbc_handle h, double* out);
  * library's kernel.
  * Its shell sums use atomic additions, so their last bits depend on the
  * order of the additions.  Device scratch (the velocity staging for host
- * input, the complex field, cuFFT's work area) comes from the allocator set
- * with kbc_set_allocator (default cudaMalloc) and is released before the
- * call returns.  Errors: KBC_ERR_ARG, KBC_ERR_NOMEM, KBC_ERR_CUDA (message:
+ * input, the complex field, cuFFT's work area; half spectra of one component
+ * at a time, half as much, where the allocator has no room for the complex
+ * field) comes from the allocator set with kbc_set_allocator (default
+ * cudaMalloc) and is released before the call returns.  Errors: KBC_ERR_ARG, KBC_ERR_NOMEM, KBC_ERR_CUDA (message:
  * kbc_last_error(NULL)). */
 int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* stream);
 

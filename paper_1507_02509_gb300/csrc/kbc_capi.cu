@@ -1699,6 +1699,7 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
         int k = 0;
         PlanPool<PoolRuntime>::Entry fft;
         bool planned = false;
+        cufftHandle real = 0;  // the plan of the real transforms
         void* get(size_t bytes)
         {
             if (bytes == 0) bytes = 256;
@@ -1715,11 +1716,18 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
         {
             cudaStreamSynchronize(s);
             if (planned) g_plans.put(fft);
-            for (int j = 0; j < k; ++j) {
-                if (al.release) al.release(p[j], (void*)s, al.user);
-                else cudaFree(p[j]);
-            }
+            if (real) cufftDestroy(real);
+            release(0);
             cudaGetLastError();
+        }
+        // the pieces after the first `keep`, which no work uses any more
+        void release(int keep)
+        {
+            while (k > keep) {
+                --k;
+                if (al.release) al.release(p[k], (void*)s, al.user);
+                else cudaFree(p[k]);
+            }
         }
     } sc{al, s};
     const size_t nn = (size_t)n * n;
@@ -1731,31 +1739,55 @@ int kbc_spectrum(int n, const double* u, int nbins, double* E, double* Z, void* 
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "spectrum: upload");
         du = st;
     }
-    double2* uh = static_cast<double2*>(sc.get(nn * sizeof(double2)));
     double* acc = static_cast<double*>(sc.get(2 * (size_t)nbins * sizeof(double)));
-    if (!uh || !acc) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: scratch allocation failed");
-    // cuFFT (a library step) with its work area from the same allocator
+    if (!acc) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: scratch allocation failed");
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (!g_plans.get(n, &sc.fft)) return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT plan");
-    sc.planned = true;
-    void* work = sc.get(sc.fft.work);
-    if (!work) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: cuFFT work area allocation failed");
-    if (cufftSetWorkArea(sc.fft.plan, work) != CUFFT_SUCCESS || cufftSetStream(sc.fft.plan, s) != CUFFT_SUCCESS)
-        return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT work area / stream");
     cudaError_t e = cudaMemsetAsync(acc, 0, (size_t)nbins * sizeof(double), s);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "spectrum: memset");
     const size_t smem = (size_t)nbins * sizeof(double);
     const int use_smem = smem <= (size_t)160 * 1024 ? 1 : 0;
-    if (use_smem && smem > 48 * 1024)
-        cudaFuncSetAttribute(spectrum_bin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (use_smem && smem > 48 * 1024) {
+        cudaFuncSetAttribute(spectrum_bin<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(spectrum_bin<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
     const double scale = 1.0 / ((double)nn * (double)nn);
-    spectrum_pack<<<sms * 8, 256, 0, s>>>(du, (long long)nn, uh);
-    if (cufftExecZ2Z(sc.fft.plan, reinterpret_cast<cufftDoubleComplex*>(uh), reinterpret_cast<cufftDoubleComplex*>(uh),
-                     CUFFT_FORWARD) != CUFFT_SUCCESS)
-        return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT execution");
-    spectrum_bin<<<sms * 4, 256, use_smem ? smem : 0, s>>>(uh, n, nbins, scale, acc, use_smem);
+    // cuFFT (a library step) with its work area from the same allocator: one
+    // complex transform of both components, or, where there is no room for it
+    // (32 n^2 bytes with its work area), one real transform after the other
+    // (half of that)
+    const int before = sc.k;
+    double2* uh = static_cast<double2*>(sc.get(nn * sizeof(double2)));
+    sc.planned = uh && g_plans.get(n, &sc.fft);
+    void* work = sc.planned ? sc.get(sc.fft.work) : nullptr;
+    if (work) {
+        if (cufftSetWorkArea(sc.fft.plan, work) != CUFFT_SUCCESS || cufftSetStream(sc.fft.plan, s) != CUFFT_SUCCESS)
+            return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT work area / stream");
+        spectrum_pack<<<sms * 8, 256, 0, s>>>(du, (long long)nn, uh);
+        if (cufftExecZ2Z(sc.fft.plan, reinterpret_cast<cufftDoubleComplex*>(uh),
+                         reinterpret_cast<cufftDoubleComplex*>(uh), CUFFT_FORWARD) != CUFFT_SUCCESS)
+            return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT execution");
+        spectrum_bin<false><<<sms * 4, 256, use_smem ? smem : 0, s>>>(uh, n, nbins, scale, acc, use_smem);
+    } else {
+        sc.release(before);
+        size_t ws = 0;
+        uh = static_cast<double2*>(sc.get((size_t)n * (n / 2 + 1) * sizeof(double2)));
+        if (!uh) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: scratch allocation failed");
+        if (cufftCreate(&sc.real) != CUFFT_SUCCESS) return fail(nullptr, KBC_ERR_CUDA, "spectrum: cufftCreate");
+        if (cufftSetAutoAllocation(sc.real, 0) != CUFFT_SUCCESS ||
+            cufftMakePlan2d(sc.real, n, n, CUFFT_D2Z, &ws) != CUFFT_SUCCESS)
+            return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT plan");
+        if (!(work = sc.get(ws))) return fail(nullptr, KBC_ERR_NOMEM, "spectrum: cuFFT work area allocation failed");
+        if (cufftSetWorkArea(sc.real, work) != CUFFT_SUCCESS || cufftSetStream(sc.real, s) != CUFFT_SUCCESS)
+            return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT work area / stream");
+        for (int c = 0; c < 2; ++c) {
+            if (cufftExecD2Z(sc.real, const_cast<double*>(du) + c * nn, reinterpret_cast<cufftDoubleComplex*>(uh)) !=
+                CUFFT_SUCCESS)
+                return fail(nullptr, KBC_ERR_CUDA, "spectrum: cuFFT execution");
+            spectrum_bin<true><<<sms * 4, 256, use_smem ? smem : 0, s>>>(uh, n, nbins, scale, acc, use_smem);
+        }
+    }
     spectrum_enstrophy<<<(nbins + 255) / 256, 256, 0, s>>>(acc, acc + nbins, nbins, n);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(E, acc, (size_t)nbins * sizeof(double), cudaMemcpyDefault, s);

@@ -32,8 +32,11 @@ __device__ __forceinline__ int shell_of(int m)
 // shell changes; a warp in one shell adds once.  (One atomic addition and one
 // double square root per coefficient took as long as a transform.)  With
 // smem != 0 a block sums in a shared histogram of nbins doubles first.
+// HALF: z is the half spectrum of a real field, columns 0 .. n/2, of which those
+// between stand for their Hermitian partners as well.
 constexpr int kShellRun = 8;
 
+template <bool HALF>
 __global__ void __launch_bounds__(256)
 spectrum_bin(const double2* __restrict__ z, int n, int nbins, double scale, double* __restrict__ E, int smem)
 {
@@ -46,19 +49,20 @@ spectrum_bin(const double2* __restrict__ z, int n, int nbins, double scale, doub
     auto put = [&](int shell, double v) {
         if (shell < nbins) atomicAdd(sum + shell, v * (0.5 * scale));
     };
-    const int lane = threadIdx.x & 31, chunks = (n + 32 * kShellRun - 1) / (32 * kShellRun);
+    const int w = HALF ? n / 2 + 1 : n;  // columns
+    const int lane = threadIdx.x & 31, chunks = (w + 32 * kShellRun - 1) / (32 * kShellRun);
     const int warps = gridDim.x * (blockDim.x >> 5);
     for (long long t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < (long long)n * chunks; t += warps) {
         const int ky = (int)(t / chunks), x0 = ((int)(t - (long long)ky * chunks) * 32 + lane) * kShellRun;
         const int fy = 2 * ky < n ? ky : ky - n;
-        const double2* row = z + (long long)ky * n;
+        const double2* row = z + (long long)ky * w;
         double acc = 0.0;
         int cur = -1;
         bool moved = false;
 #pragma unroll
         for (int j = 0; j < kShellRun; ++j) {
             const int kx = x0 + j;
-            if (kx >= n) break;
+            if (kx >= w) break;
             const int fx = 2 * kx < n ? kx : kx - n;
             const int shell = shell_of(fx * fx + fy * fy);
             if (shell != cur && cur >= 0) {
@@ -68,7 +72,8 @@ spectrum_bin(const double2* __restrict__ z, int n, int nbins, double scale, doub
             }
             cur = shell;
             const double2 c = row[kx];
-            acc = fma(c.x, c.x, fma(c.y, c.y, acc));
+            if constexpr (HALF) acc = fma(kx == 0 || 2 * kx == n ? 1.0 : 2.0, fma(c.x, c.x, c.y * c.y), acc);
+            else acc = fma(c.x, c.x, fma(c.y, c.y, acc));
         }
         const int first = __shfl_sync(0xffffffffu, cur, 0);
         if (__all_sync(0xffffffffu, !moved && cur == first)) {
