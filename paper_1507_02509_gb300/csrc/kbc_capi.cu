@@ -1298,20 +1298,23 @@ int kbc_adjoint(kbc_handle h, const double* rho0, const double* u0, int nsteps, 
     // ten took 10 us through the caller's allocator, half of what a step of
     // a 512^2 grid takes): inputs rho0, u0 and the target; dJ/du0; sums; two
     // fields, two lambdas; one bit per node for the single-precision reverse
-    // steps left to the double redo; a copy of a checkpoint
+    // steps left to the double redo; a copy of a checkpoint.  An allocator
+    // that has no piece of that size is asked for the parts, of which the last
+    // only saves launches.
     const bool even = K % 2 == 0 && h->graph_steps > 0;
     const size_t maskbytes = (size_t)((n + 31) / 32) * sizeof(unsigned);
     const size_t sizes[] = {(size_t)(objective == 1 ? 5 : 3) * n * sizeof(double), (size_t)2 * n * sizeof(double),
                             (size_t)(2 * nb + 8) * sizeof(double), field, field, lamf, lamf, maskbytes,
                             even && nsteps / K >= 2 ? field : 0};
-    void* piece[9];
+    void* piece[9] = {};
     size_t bytes = 0;
     for (size_t b : sizes) bytes += (b + 255) & ~(size_t)255;
     char* arena = static_cast<char*>(B.get(bytes));
-    if (!arena) return fail(h, KBC_ERR_NOMEM, "adjoint buffers");
     for (int k = 0; k < 9; ++k) {
-        piece[k] = arena;
-        arena += (sizes[k] + 255) & ~(size_t)255;
+        if (sizes[k] == 0) continue;
+        piece[k] = arena ? arena : B.get(sizes[k]);
+        if (!piece[k] && k < 8) return fail(h, KBC_ERR_NOMEM, "adjoint buffers");
+        if (arena) arena += (sizes[k] + 255) & ~(size_t)255;
     }
     double* in = static_cast<double*>(piece[0]);
     double* gdev = static_cast<double*>(piece[1]);
@@ -1319,7 +1322,7 @@ int kbc_adjoint(kbc_handle h, const double* rho0, const double* u0, int nsteps, 
     void* work[2] = {piece[3], piece[4]};
     void* lam[2] = {piece[5], piece[6]};
     unsigned* fixmask = static_cast<unsigned*>(piece[7]);
-    void* ckwork = sizes[8] ? piece[8] : nullptr;
+    void* ckwork = piece[8];
     // checkpoints and segment states in two slabs
     char* ckslab = nseg ? static_cast<char*>(B.get(field * (size_t)nseg)) : nullptr;
     char* segslab = seglen > 1 ? static_cast<char*>(B.get(field * (size_t)(seglen - 1))) : nullptr;
@@ -1335,7 +1338,7 @@ int kbc_adjoint(kbc_handle h, const double* rho0, const double* u0, int nsteps, 
     // float B, 100 steps in one segment: 3.8 -> 1.9 ms with both.
     AdjointGraphs G;
     const int last0 = nseg > 0 ? (nseg - 1) * K : 0;  // first step of the last segment
-    const bool fwd_graphs = even && nseg - 1 >= 2;    // every segment before the last is full
+    const bool fwd_graphs = ckwork && nseg - 1 >= 2;    // every segment before the last is full
     const bool graphs = ckwork != nullptr;
     cudaError_t e = cudaMemcpyAsync(in, rho0, n * sizeof(double), cudaMemcpyDefault, h->stream);
     if (e == cudaSuccess)
