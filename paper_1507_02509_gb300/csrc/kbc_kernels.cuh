@@ -972,14 +972,22 @@ __device__ __forceinline__ void diag_ext_fold(double* a, int sa, const double* b
     a[0] = na + nb;
 }
 
+// The library's logarithm out of line: code that hardly any node takes should
+// not cost the others registers.
+static __device__ __noinline__ double log1p_one(double x) { return log1p(x); }
+
+// Bound by the FP64 pipe (4096^2 float 10.3 ms with the library's logarithm and
+// an IEEE division per moment, 4.1 ms now).  Four blocks per SM, all of the
+// grid: 64 registers, of which doubles spill 116 bytes; with 78 and three
+// blocks the fourth quarter of the grid runs alone (1024^2 float 324 -> 411 us).
 template <class C>
-__global__ void __launch_bounds__(kDiagBlock)
+__global__ void __launch_bounds__(kDiagBlock, 4)
 diag_ext_partial(const typename C::S* __restrict__ src, double* __restrict__ part, StepArgs a)
 {
     // u on the tile with a two-node halo, w on the tile with a one-node halo
     constexpr int UW = kTileW + 4, UH = kTileH + 4, WW = kTileW + 2, WH = kTileH + 2;
     __shared__ double sux[UH][UW], suy[UH][UW], sw[WH][WW];
-    __shared__ EntropyTable logs;
+    __shared__ EntropyLogs logs;
     logs.fill();
     double acc[kDiagExtParts] = {0, 0, 0, 0, 0};  // n, mean and M2 of P, of s
     const int ntx = (a.nx + kTileW - 1) / kTileW, nty = (a.ny + kTileH - 1) / kTileH;
@@ -1002,36 +1010,42 @@ diag_ext_partial(const typename C::S* __restrict__ src, double* __restrict__ par
         __syncthreads();
         for (int k = threadIdx.x; k < kTileW * kTileH; k += blockDim.x) {
             const int ly = k / kTileW, lx = k - ly * kTileW;
-            const int x = x0 + lx, y = y0 + ly;
-            if (x >= a.nx || y >= a.ny) continue;
+            const int xn = x0 + lx, y = y0 + ly;
+            if (xn >= a.nx || y >= a.ny) continue;
             const int cx = lx + 1, cy = ly + 1;
             const double wx = 0.5 * (sw[cy][cx + 1] - sw[cy][cx - 1]);
             const double wy = 0.5 * (sw[cy + 1][cx] - sw[cy - 1][cx]);
             const double pp = 0.5 * (wx * wx + wy * wy);
-            const long long n = (long long)y * a.nx + x;
-            // s = -sum W_i (1 + x_i) ln(1 + x_i), x_i = d_i / W_i, by weight class
+            const long long n = (long long)y * a.nx + xn;
+            // s = -sum W_i (1 + x_i) ln(1 + x_i), x_i = d_i / W_i
             typename C::S raw[9];
-            double xs[9];
-            float xf[9];
+            double x[9], se = 0.0;
             bool near = true;
 #pragma unroll
             for (int i = 0; i < 9; ++i) raw[i] = src[(long long)i * a.plane + n];
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                xs[i] = C::to_f64(raw[i], i, a.cs) * inv_wgt(i);
-                xf[i] = leading(xs[i]);
-                near &= fabsf(xf[i]) < 0.5f;
+                x[i] = C::relative(raw[i], i, a.cs);
+                near &= (__double2hiint(x[i]) & 0x7fffffff) < 0x3fe00000;  // |x| < 1/2
             }
-            double se = 0.0;
             if (near) {
+                // sums by weight class; the weights are 1, 4 and 16 times 1/36
                 double sum[3] = {0.0, 0.0, 0.0};
+                long long units = 0;
 #pragma unroll
-                for (int i = 0; i < 9; ++i)
-                    sum[wclass(i)] += logs.entropy_near(xs[i], xf[i]);
-                se = -__fma_rn(wgt(0), sum[0], __fma_rn(wgt(1), sum[1], wgt(4) * sum[2]));
+                for (int i = 0; i < 9; ++i) {
+                    long long unit;
+                    sum[wclass(i)] += logs.near(x[i], leading(x[i]), unit);
+                    units += unit << (2 * wclass(i));
+                }
+                se = -__fma_rn(EntropyLogs::as_double(units), 0x1p-46 * wgt(0),
+                               __fma_rn(wgt(0), sum[0], __fma_rn(wgt(1), sum[1], wgt(4) * sum[2])));
             } else {
 #pragma unroll
-                for (int i = 0; i < 9; ++i) se -= wgt(i) * (1.0 + xs[i]) * log1p(xs[i]);
+                for (int i = 0; i < 9; ++i) {
+                    const double d = C::to_f64(src[(long long)i * a.plane + n], i, a.cs);
+                    se -= (wgt(i) + d) * log1p_one(d * inv_wgt(i));
+                }
             }
             acc[0] += 1.0;
             const double rn = rcp_pos(acc[0]);

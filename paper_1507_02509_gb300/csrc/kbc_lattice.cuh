@@ -159,6 +159,8 @@ struct CodecF64 {
     __device__ __forceinline__ static T load(S s, int, const CodecScale&) { return s; }
     __device__ __forceinline__ static S store(T d, int, const CodecScale&) { return d; }
     __device__ __forceinline__ static double to_f64(S s, int, const CodecScale&) { return s; }
+    // d_i / W_i in double
+    __device__ __forceinline__ static double relative(S s, int i, const CodecScale&) { return s * inv_wgt(i); }
     __device__ __forceinline__ static S from_f64(double d, int, const CodecScale&) { return d; }
 };
 
@@ -172,6 +174,7 @@ struct CodecF32 {
     __device__ __forceinline__ static T load(S s, int, const CodecScale&) { return s; }
     __device__ __forceinline__ static S store(T d, int, const CodecScale&) { return d; }
     __device__ __forceinline__ static double to_f64(S s, int, const CodecScale&) { return widen(s); }
+    __device__ __forceinline__ static double relative(S s, int i, const CodecScale&) { return widen(s) * inv_wgt(i); }
     __device__ __forceinline__ static S from_f64(double d, int, const CodecScale&) { return narrow(d); }
 };
 
@@ -205,6 +208,10 @@ struct CodecF16 {
     __device__ __forceinline__ static double to_f64(S s, int i, const CodecScale& c)
     {
         return widen(__half2float(__ushort_as_half(s))) * (wgt(i) * (double)c.inv_scale);
+    }
+    __device__ __forceinline__ static double relative(S s, int, const CodecScale& c)
+    {
+        return widen(__half2float(__ushort_as_half(s))) * (double)c.inv_scale;
     }
     __device__ __forceinline__ static S from_f64(double d, int i, const CodecScale& c)
     {
