@@ -97,8 +97,11 @@ static __device__ __noinline__ double divide_one(double x) { return 1.0 / x; }
 // 1 / x in double for positive normal x (others by the IEEE division): with
 // x = m 2^k, 1 <= m < 2, the single-precision reciprocal y of m's leading bits
 // (relative error below 2^-21), then y (1 + r + r^2) with the residual
-// r = 1 - m y, whose remainder r^3 is below the last bit.  Three FP64
-// instructions; the IEEE division takes about nine.
+// r = 1 - m y, whose remainder r^3 is below the last bit: one value in a million
+// rounds otherwise than the quotient (30 of 3.4e7, none by more than one unit;
+// a refinement of y in single precision made that fewer for random values and
+// more, 6.6e4, for those next to powers of two, where the quotients are nearly
+// ties).  Three FP64 instructions; the IEEE division takes about nine.
 __device__ __forceinline__ double rcp_pos(double x)
 {
     const unsigned H = (unsigned)__double2hiint(x), B = (unsigned)__double2loint(x);
