@@ -190,9 +190,10 @@ int kbc_set_gamma_mode(kbc_handle h, int mode, double gamma_fixed);
  *   KBC_KERNEL_AUTO  (default) the fastest choice measured on GB300: the
  *                    per-node kernel for F64, for KBC variants on small grids
  *                    and for widths the others do not take; the bulk-copy
- *                    kernel below for F16 storage with A or B on large
- *                    grids with nx a multiple of 512; otherwise the vector-row
- *                    kernel where nx is a multiple of its row width;
+ *                    kernel below, with nx a multiple of 512, for F16 storage
+ *                    with A or B where both fields exceed 100 MB and with
+ *                    LBGK where they take 80 to 240 MB; otherwise the
+ *                    vector-row kernel where nx is a multiple of its row width;
  *   KBC_KERNEL_ROWS  the vector-row kernel where nx allows it, else the
  *                    per-node kernel;
  *   KBC_KERNEL_NODES the per-node kernel;

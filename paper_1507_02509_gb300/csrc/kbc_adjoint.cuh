@@ -46,7 +46,7 @@ template <int VAR, typename T> constexpr int adj_min_blocks()
 // products, their adjoints) is one packed operation for two populations,
 // with sign pairs (a, -a), (b, -b) for the velocity components; the rest
 // population i = 4 and the scalar moments stay scalar.  Same mathematics as
-// the generic collide_adjoint below, in a different rounding order.
+// collide_adjoint below, the one in double, in a different rounding order.
 template <int VAR>
 __device__ __forceinline__ bool collide_adjoint_pairs(const float (&d)[9], const float (&lam)[9],
                                                       const CollideParams<float>& p,
@@ -56,7 +56,7 @@ __device__ __forceinline__ bool collide_adjoint_pairs(const float (&d)[9], const
     constexpr bool central = (VAR == kA || VAR == kB);
     bool guarded = false;
     // ---------------------------------------------------------------- forward
-    // the pairwise moment sums of the generic path
+    // the pairwise moment sums of collide_adjoint
     const float drho = ((d[0] + d[8]) + (d[2] + d[6])) + ((d[1] + d[7]) + (d[3] + d[5])) + d[4];
     const float jx = ((d[2] - d[0]) + (d[8] - d[6])) + (d[5] - d[3]);
     const float jy = ((d[6] - d[0]) + (d[8] - d[2])) + (d[7] - d[1]);

@@ -404,17 +404,21 @@ static int step_into(kbc_handle h, const void* src, void* dst, cudaStream_t stre
     Launch L;
     L.variant = h->variant;
     // AUTO takes, measured in us a step with the others in brackets:
-    // - per node for doubles (64^2 B 8.1 [rows 14.5], 2048^2 1525 [1541]), for
+    // - per node for doubles (64^2 B 7.8 [rows 13.9], 2048^2 1486 [1503]), for
     //   KBC on grids whose nodes are all resident at once (256^2 F32 B 3.1
-    //   [rows 3.4]; F16 B 2.1 [rows 2.25]) and for the widths that the other
-    //   two do not take;
-    // - bulk copies for FP16 A and B beyond L2 (4096^2 B 136 [rows 137];
-    //   1536^2 19.4 for the rows [bulk 20.4]);
+    //   [rows 3.3]; F16 B 2.2 [2.1]) and for the widths that the other two do
+    //   not take;
+    // - bulk copies for FP16 A and B beyond L2 (B, rows over bulk: 78 MB 0.91,
+    //   94 MB 0.96, 113 MB 1.005, 151 MB 1.016, 340 MB 1.013; 4096^2 135.0
+    //   [136.7]);
     // - bulk copies for FP16 LBGK on fields about the size of L2, 80 to 240 MB
-    //   (1536^2 11.4 [rows 12.8], 2048^2 20.7 [27.8]; 1024^2 6.5 [6.2], 3072^2
-    //   63 [59]);
-    // - vector rows otherwise (4096^2 F32 B 180 [bulk 221], LBGK 172 [196],
+    //   (rows over bulk: 66 MB 0.95, 78 MB 1.00, 85 MB 1.03, 151 MB 1.12, 236 MB
+    //   1.06, 340 MB 1.03; 4096^2, 604 MB, 0.96);
+    // - vector rows otherwise (4096^2 F32 B 177 [bulk 213], LBGK 168 [193],
     //   F16 C 122 [bulk 126]).
+    // A y-slab counts by its own size, also where a grid is stepped slab after
+    // slab: by the grid's size LBGK and B of float gained 1%, but half lost 4 to
+    // 10% (2048 x 1536 in four, B: 34.0 us a step, 37.5 by the grid's size).
     const long long total = (long long)h->nx * h->ny;
     const bool tiles = h->dtype != KBC_F64 && h->nx % kTmaTile == 0, kbc = h->variant != KBC_LBGK;
     const bool autok = h->kernel == KBC_KERNEL_AUTO || (h->kernel == KBC_KERNEL_BULK && !tiles);
@@ -1660,7 +1664,7 @@ int kbc_slabs_step(int parts, const kbc_handle* slabs, int nsteps)
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "slab halos");
         const int back = hs[0]->sweep;
         for (int k = 0; k < parts; ++k) {
-            kbc_handle h = hs[back ? parts - 1 - k : k];  // one sweep over the whole grid
+            kbc_handle h = hs[back ? parts - 1 - k : k];  // from the end that was written last
             h->sweep = back;
             h->ghosts_full = 0;
             const int rc = step_into(h, h->buf[h->cur], h->buf[h->cur ^ 1]);

@@ -190,13 +190,19 @@ __device__ __forceinline__ bool collide_settled(const float (&d)[9], const Guard
     const Lf sh = fmaL(Lf(13.5f), s0a + s0b, fmaL(Lf(20.25f), s0c, -s1));
     const Lf R = ratio(sh, hh), nb(p.nb);
     const Lf nch = fmaL(nb, R, nb);
-    // Error bound.  delta: the moments of df, from the products (three pair
-    // products of 2^-45 and the rounding of the differences) and, 2^-50 of
-    // the largest value, from the double computation that this stands for; the
-    // populations made of them are off by at most 3 delta, times 1/4 and 1/2
-    // on the diagonals and axes.  us, uh: rounding of ds and dh formed from
-    // their moments.  The sums' own rounding is 14 u of their magnitudes,
-    // where |P / (1 + P)| <= 1.5 pm.
+    // Error bound.  delta: the moments of df.  1 / rho is a pair to 2^-46, u to
+    // 2^-44.3, a product rho u u to 2^-43.6 (M22 holds a third of two of them,
+    // the third moments hold none and are far more exact), and the double
+    // computation that this stands for adds 2^-50 of the largest value.  The
+    // split adds um < 0.3 times delta to third and um^2 to fourth moments, so
+    // that the populations made of the moments are off by at most 3 delta,
+    // times 1/4 and 1/2 on the diagonals and axes (at rest three moments enter
+    // whole, of which M22 with a third).  us, uh: rounding of ds and dh formed
+    // from their moments.  The sums' own rounding is 14 u of their magnitudes:
+    // nine additions, two products and three for the weight, where
+    // |P / (1 + P)| <= pm.  <ds|dh>'s part under 1 / W moves with the errors of
+    // f22 and g22, below 1.7 delta (20.25 of it, 35), and with those of the
+    // third moments, below 2 um delta (13.5 of it 27 um; 60 um is taken).
     const float u = 0x1p-24f;
     const float delta = 0x1p-43f * (mxx.h.v + myy.h.v) + __uint_as_float((unsigned)(e - 49) << 23);
     const float um = fabsf(ux.h.v) + fabsf(uy.h.v), pm = 1.5f * (3.0f * um + 6.0f * um * um);

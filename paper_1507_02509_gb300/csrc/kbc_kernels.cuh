@@ -239,8 +239,9 @@ __device__ __forceinline__ unsigned collide_vec(T (&f)[NV][9], const CollidePara
 // nbx * ny blocks, nbx = ceil(nx / (BLOCK NV)) blocks per row; warps past
 // the row end exit as a whole.
 // PAIRS: the four nodes are collided as two packed lane pairs, which takes 40%
-// fewer instructions and up to 128 registers: 8 resident blocks per SM (10 for
-// the natural-basis variants and LBGK, whose pairs fit 96) instead of 12.
+// fewer instructions and up to 128 registers: 8 resident blocks per SM (10, of
+// 96 registers, for the natural-basis variants and LBGK) instead of 12.  Half
+// storage fits them; float spills 4 bytes (A), 12 (B), 32 (C) and 48 (D).
 // That is the faster side where instructions bound the step: half storage
 // (4096^2 C 143 -> 122 us, bulk copies 126; 1024^2 B 10.5 -> 9.5), and
 // float fields that stay in L2 (1024^2 B 12.2 -> 11.6, C 11.4 -> 10.8);
@@ -342,14 +343,15 @@ step_rows(const typename C::S* __restrict__ src, typename C::S* __restrict__ dst
 // nodes lie in one row, away from its ends, addresses every population as
 // one offset shared by the warp plus the thread's index; the others wrap per
 // thread.  Bound by the latency of the collision: K = 4 gives it two
-// independent pairs (4095 x 4096, float B: K = 4 193 us, K = 2 248 us, one
-// node at a time 237 us; one node per thread with a 64-bit division before,
-// 281 us); float C needs 94 registers and runs at the copy bandwidth with
-// ten blocks per SM (176 us against 189 us with eight).  A grid whose nodes
-// find a thread each at once takes K = 1 (256^2, float B: 3.5 us a step
-// against 3.8 for the vector rows).  Double is bound by the FP64 pipe and
-// takes K = 1 everywhere (64^2: 8.1 us against 14.5 with the two nodes a
-// thread of the vector rows, 2048^2 1525 against 1541 us).
+// independent pairs (4095 x 4096, float B, all sweeps in one direction: K = 4
+// 193 us, K = 2 248 us, one node at a time 237 us; one node per thread with a
+// 64-bit division before, 281 us; 185 us with alternating sweeps); float C
+// needs 94 registers and runs at the copy bandwidth with ten blocks per SM (176
+// us against 189 us with eight), half C spills 64 bytes there.  A grid whose
+// nodes find a thread each at once takes K = 1 (256^2, float B: 3.1 us a step
+// against 3.3 for the vector rows).  Double is bound by the FP64 pipe and takes
+// K = 1 everywhere (64^2: 7.8 us against 13.9 with the two nodes a thread of
+// the vector rows, 2048^2 1486 against 1503 us).
 constexpr int kFlatBlock = 64;
 // Nodes per thread on a grid that fills the GPU, and resident blocks per SM
 // the kernel is compiled for.
@@ -550,10 +552,11 @@ __device__ __noinline__ void feq_node_general(double r, double x, double y,
 // storage in pairs of floats, packed over the nodes: the moment form of
 // feq_node with the factors 1/9, 1/3 and 1 (float) or S, 3 S and 9 S (half
 // codes are (f - W) S / W) on q, the first- and second-order terms.  Error
-// bound: every term is a product of at most four pairs (4 2^-45) of inputs
-// with 2^-48, then at most four additions (2^-46 of M each), so 2^-42 M
-// covers it, M the sum of the terms' magnitudes (for the rest population
-// its own two terms'); the double computation's own error is 2^-50 M.
+// bound, relative: the inputs 2^-48, rho 2^-47, a product 2^-45 more (see
+// FF), so j 2^-44.5, and A, B and C9, of three more factors, 2^-43.3; then at
+// most four additions, 2^-46 of M each, M the sum of the terms' magnitudes (for
+// the rest population its own two terms').  2^-42.7 in all, of which 2^-42 M
+// leaves a third, and the double computation's own error is 2^-50 M.
 template <class C>
 __device__ __forceinline__ void feq_pair(const double (&r)[2], const double (&x)[2], const double (&y)[2],
                                          typename C::S* __restrict__ dst, long long n0, long long n1,

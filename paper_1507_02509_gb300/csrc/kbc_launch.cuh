@@ -27,8 +27,9 @@ enum class StepKind { rows, nodes, bulk };
 inline bool flat_small(int nx, int ny, int num_sms) { return (long long)nx * ny <= (long long)num_sms * 1024; }
 
 // Whether the two fields of a step stay in L2 (129 MB, of which 100 MB hold
-// them without the rest of the step pushing them out: 1024^2 float, 75 MB, is
-// inside, 1536^2, 170 MB, outside).
+// them without the rest of the step pushing them out: what half B gains by the
+// kernels for either side changes sign between 94 and 113 MB; 1024^2 float, 75
+// MB, is inside, 1536^2, 170 MB, outside).
 inline bool rows_in_l2(long long total, size_t elem) { return 18.0 * (double)elem * (double)total <= 100e6; }
 
 struct Launch {
