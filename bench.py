@@ -85,10 +85,12 @@ def step_kernel_name(args) -> str:
     return {"rows": "step_rows", "bulk": "step_tma", "nodes": "step_nodes"}[k]
 
 
-def kernel_source_hash() -> str:
-    """Hash of the code that defines the vector-row step kernel: the lattice,
-    lane and collision headers, the kernel's own section of kbc_kernels.cuh
-    and its launch width."""
+def kernel_source_hash(kernel: str = "step_rows") -> str:
+    """Hash of the code that defines the vector-row step kernel (or the
+    per-node one, "step_nodes"): the lattice, lane and collision headers, the
+    kernel's own section of kbc_kernels.cuh and its launch width."""
+    first, last, width = {"step_rows": ("step, rows", "step, nodes", "kRowBlock"),
+                          "step_nodes": ("step, nodes", "all-FP64 step", "kFlatBlock")}[kernel]
     csrc = os.path.join(ROOT, "paper_1507_02509_gb300", "csrc")
     h = hashlib.sha256()
     for name in ("kbc_lattice.cuh", "kbc_lanes.cuh", "kbc_collide.cuh"):
@@ -96,11 +98,11 @@ def kernel_source_hash() -> str:
             h.update(name.encode() + f.read())
     with open(os.path.join(csrc, "kbc_kernels.cuh")) as f:
         text = f.read()
-    a = text.index("// ---------------------------------------------------------------- step, rows")
-    b = text.index("// ---------------------------------------------------------------- step, nodes")
+    a = text.index("// ---------------------------------------------------------------- " + first)
+    b = text.index("// ---------------------------------------------------------------- " + last)
     h.update(text[a:b].encode())
     with open(os.path.join(csrc, "kbc_launch.cuh")) as f:
-        h.update("".join(l for l in f if "kRowBlock" in l).encode())
+        h.update("".join(l for l in f if width in l).encode())
     return h.hexdigest()[:16]
 
 
@@ -472,7 +474,7 @@ def run_ours(args):
         # measured DFMA issue rate, its use the FP64 thread-instructions per
         # node (ncu, profiles/) at the measured update rate
         rate = capi.kbc_fp64_fma_rate(ctypes.c_void_p(stream.cuda_stream))
-        ops = fp64_ops_from_profile("step_rows<B,f64>") if args.variant == "B" else None
+        ops = fp64_ops_from_profile("step_nodes<B,f64>") if args.variant == "B" else None
         if "f64" in extras:
             extras["f64"]["fp64_dfma_per_s"] = rate
             extras["f64"]["fp64_inst_per_node"] = ops
@@ -653,7 +655,8 @@ def fp64_ops_from_profile(kernel: str):
     """FP64 thread-instructions per node of the FP64 step kernel from the
     committed ncu summary, or None when missing, taken on another kernel or
     on other sources."""
-    path = os.path.join(ROOT, "profiles", "kbc_step_rows_f64_ops.txt")
+    name = kernel.split("<")[0]
+    path = os.path.join(ROOT, "profiles", f"kbc_{name}_f64_ops.txt")
     if not os.path.exists(path):
         return None
     vals = {}
@@ -663,7 +666,7 @@ def fp64_ops_from_profile(kernel: str):
                 k, v = line.split(":", 1)
                 vals[k.strip()] = v.strip()
     try:
-        if vals.get("kernel_source_hash") != kernel_source_hash() or vals.get("kernel") != kernel:
+        if vals.get("kernel_source_hash") != kernel_source_hash(name) or vals.get("kernel") != kernel:
             return None
         return float(vals["fp64_inst_per_node"])
     except (KeyError, ValueError):
