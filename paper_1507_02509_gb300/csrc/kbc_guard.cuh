@@ -233,12 +233,16 @@ __device__ __forceinline__ bool collide_settled(const float (&d)[9], const Guard
 // One block of 16 warps per SM.  A list of up to 128 nodes per block is
 // collided in double at once: one warp per scheduler, whose 220 instructions
 // of 64 cycles are the shortest time a double collision takes (7 us).  A
-// longer one is cut into a stretch per block and warp; each warp works
-// through its own and leaves the nodes that are not settled at the stretch's
-// beginning, and after one block barrier the block collides those in double.
-// 1024^2 shear layer, B, steps 92 to 156 (250 to 400 k nodes a step): 231 us
-// a step with the double collision of every node and an atomic addition per
-// lane that reports one, 67 us now, of which 12 are the step's.
+// longer one is dealt out in pieces of 32 entries, first over the blocks, then
+// over their warps, so that lists of any length and nodes of either kind, which
+// lie together, come evenly to the SMs; each warp works through its own pieces
+// and leaves the nodes that are not settled at the beginning of them, and after
+// one block barrier the block collides those in double.  A warp that settles
+// fewer than a quarter leaves its other pieces as they are.
+// 1024^2, float B, us a step with every node in double and an atomic addition
+// per lane that reports one, with a stretch of the list per block, and now:
+// shear layer at 200 steps 151, 45, 39; a vortex with 27 k nodes 29, 50, 28; at
+// rest, where nothing is settled, 471, 488, 449.
 constexpr int kGuardBlock = 512;
 constexpr int kGuardWarps = kGuardBlock / 32;
 constexpr int kGuardDirect = 128;
@@ -247,7 +251,9 @@ template <int VAR>
 __global__ void __launch_bounds__(kGuardBlock, 1)
 step_guard(const float* __restrict__ src, float* __restrict__ dst, StepArgs a, GuardParams gp)
 {
-    __shared__ int left[kGuardWarps];
+    // per warp: entries left, and those of them at the beginning of its
+    // pieces; the others are all from the piece `from` on
+    __shared__ int left[kGuardWarps], kept_of[kGuardWarps], from_of[kGuardWarps];
     chain_enter();
     const int recorded = ld_count(a.fix_count + a.fix_slot);
     const int count = recorded < a.nx * a.ny ? recorded : a.nx * a.ny;
@@ -265,23 +271,26 @@ step_guard(const float* __restrict__ src, float* __restrict__ dst, StepArgs a, G
             f[i] = ld_field(src + (long long)i * a.plane + (long long)sy * a.nx + sx);
         }
     };
+    // place in the list of entry q of warp w's pieces
+    auto place = [&](int w, int q) {
+        return (((long long)(q >> 5) * kGuardWarps + w) * blocks + blockIdx.x) * 32 + (q & 31);
+    };
     const bool direct = !gp.settle || count <= blocks * kGuardDirect;
-    // entries per warp (a multiple of 32) and the block's first
-    const int per = (int)((((long long)count + blocks - 1) / blocks + kGuardBlock - 1) / kGuardBlock) * 32;
-    const long long t0 = (long long)blockIdx.x * per * kGuardWarps;
     int m;
     if (direct) {
         m = (count - (int)blockIdx.x + blocks - 1) / blocks;
     } else {
-        const long long w0 = t0 + (long long)warp * per;
-        int kept = 0;
-        for (int k0 = 0; k0 < per && w0 + k0 < count; k0 += 32) {
-            bool open = w0 + k0 + lane < count;
+        // the warp's entries: whole pieces but for the list's last one
+        const int pieces = (count - 1) / 32 + 1, first = warp * blocks + (int)blockIdx.x;
+        const int own = first < pieces ? (pieces - 1 - first) / (kGuardWarps * blocks) + 1 : 0;
+        int mine = own * 32;
+        if (own > 0 && place(warp, mine - 1) >= count) mine = mine - 32 + (count & 31);
+        int kept = 0, k0 = 0;
+        for (; k0 < mine && 4 * kept <= 3 * k0; k0 += 32) {
+            bool open = k0 + lane < mine;
             int n = 0;
-            if (open) n = ld_count(a.fix_list + w0 + k0 + lane);
-            // a warp that settles fewer than a quarter of its nodes leaves the
-            // rest of them as they are
-            if (open && 4 * kept <= 3 * k0) {
+            if (open) {
+                n = ld_count(a.fix_list + place(warp, k0 + lane));
                 float f[9], out[9];
                 pull(n, f);
                 open = !collide_settled<VAR>(f, gp, out);
@@ -292,10 +301,14 @@ step_guard(const float* __restrict__ src, float* __restrict__ dst, StepArgs a, G
             }
             // every lane has read its entry before entries it may overwrite
             const unsigned vote = __ballot_sync(0xffffffffu, open);
-            if (open) a.fix_list[w0 + kept + __popc(vote & ((1u << lane) - 1u))] = n;
+            if (open) a.fix_list[place(warp, kept + __popc(vote & ((1u << lane) - 1u)))] = n;
             kept += __popc(vote);
         }
-        if (lane == 0) left[warp] = kept;
+        if (lane == 0) {
+            left[warp] = kept + (k0 < mine ? mine - k0 : 0);
+            kept_of[warp] = kept;
+            from_of[warp] = k0;
+        }
         __syncthreads();  // orders the block's list entries as well
         m = 0;
 #pragma unroll
@@ -306,7 +319,7 @@ step_guard(const float* __restrict__ src, float* __restrict__ dst, StepArgs a, G
         if (!direct) {
             int w = 0, q = k;
             while (q >= left[w]) q -= left[w++];
-            t = t0 + (long long)w * per + q;
+            t = place(w, q < kept_of[w] ? q : q - kept_of[w] + from_of[w]);
         }
         const int n = ld_count(a.fix_list + t);
         float f[9];
