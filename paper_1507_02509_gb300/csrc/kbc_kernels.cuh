@@ -778,10 +778,14 @@ __device__ __forceinline__ void node_macro(const typename C::S* __restrict__ src
         FixedSums s;
         if (fixed_of<C>::sums(c, a.cs, s)) {
             rho = __fma_rn(s.unit, (double)s.drho, 1.0);
-            const double ir = rcp_pos(rho) * s.unit;
-            ux = (double)s.jx * ir;
-            uy = (double)s.jy * ir;
-            return;
+            // where rho nearly vanishes (or is negative) the rounding of the
+            // half storage's unit would be all that is left of it
+            if (__double2hiint(rho) >= 0x3eb00000) {  // 2^-20
+                const double ir = rcp_pos(rho) * s.unit;
+                ux = (double)s.jx * ir;
+                uy = (double)s.jy * ir;
+                return;
+            }
         }
     }
     double d[9];
