@@ -72,5 +72,5 @@ def test_parts_in_place_of_one_piece(dtype, steps, every, objective, last):
         lat.close()
         assert not live
     finally:
-        capi.kbc_set_allocator(capi.ALLOC_FN(0), capi.FREE_FN(0), None)
-        pkg._torch_hooks = None
+        pkg.use_torch_allocator()
+        capi.kbc_set_allocator(*pkg._torch_hooks, None)

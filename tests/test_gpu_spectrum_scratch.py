@@ -43,8 +43,8 @@ class Limited:
         import paper_1507_02509_gb300 as pkg
         from paper_1507_02509_gb300 import capi
 
-        capi.kbc_set_allocator(capi.ALLOC_FN(0), capi.FREE_FN(0), None)
-        pkg._torch_hooks = None
+        pkg.use_torch_allocator()
+        capi.kbc_set_allocator(*pkg._torch_hooks, None)
 
 
 @pytest.mark.parametrize("n", [254, 256, 510])
