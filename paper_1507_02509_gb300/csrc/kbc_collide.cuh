@@ -327,11 +327,7 @@ __device__ __forceinline__ L collide(L (&d)[9], const CollideParams<typename L::
             ds[2] = ds[6] = -q;
         }
         L dh[9];
-        if constexpr (dbl) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) dh[i] = df[i] - ds[i];
-        }
-        // the entropic weights and <ds|dh>, <dh|dh>
+        // dh, the entropic weights and <ds|dh>, <dh|dh>
         L w[9], sh, hh;
         L xprod;  // double lanes: prod_i x_i, the common factor of their weights
         auto products = [&]() {
@@ -366,7 +362,7 @@ __device__ __forceinline__ L collide(L (&d)[9], const CollideParams<typename L::
             }
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                if constexpr (!dbl) dh[i] = df[i] - ds[i];
+                dh[i] = df[i] - ds[i];
                 const L t = dh[i] * w[i];
                 if (i == 0) {
                     sh = ds[0] * t;
@@ -384,6 +380,10 @@ __device__ __forceinline__ L collide(L (&d)[9], const CollideParams<typename L::
         L nch, gamma;  // nch = -beta (gamma - 2)
         guard_hits = 0u;
         if (p.fixed) {
+            if constexpr (dbl) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) dh[i] = df[i] - ds[i];
+            }
             nch = L(-p.ch_fixed);
             gamma = L(p.gamma_fixed);
         } else {
