@@ -24,22 +24,26 @@ def test_unsettled_nodes_are_spread_over_the_blocks(rows):
     ux, uy = 0.03 * rng.standard_normal((2, n, n))
     ux[:rows] = uy[:rows] = 0.0  # at rest: <dh|dh> = 0
     g = torch.as_tensor(representable(O.init_feq(np.ones((n, n)), ux, uy), "f32")).cuda()
-    took, count, out = {}, {}, {}
+    lats = {}
     for guard in (SETTLED, DOUBLE):
-        lat = Lattice(n, n, variant="B", beta=0.985, dtype="f32")
-        lat.set_guard(guard)
-        t = []
-        for _ in range(40):
+        lats[guard] = Lattice(n, n, variant="B", beta=0.985, dtype="f32")
+        lats[guard].set_guard(guard)
+    t = {guard: [] for guard in lats}
+    for _ in range(80):  # in turn
+        for guard, lat in lats.items():
             lat.set_populations(g)
             a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
             a.record()
             lat.step(1)
             b.record()
             torch.cuda.synchronize()
-            t.append(a.elapsed_time(b))
-        took[guard], count[guard], out[guard] = float(np.median(t[8:])), lat.guard_count(), lat.populations()
+            t[guard].append(a.elapsed_time(b))
+    took = {guard: float(np.median(x[10:])) for guard, x in t.items()}
+    count = {guard: lat.guard_count() for guard, lat in lats.items()}
+    out = {guard: lat.populations() for guard, lat in lats.items()}
+    for lat in lats.values():
         lat.close()
     assert count[SETTLED] == count[DOUBLE] >= (rows - 2) * n
     assert torch.equal(out[SETTLED], out[DOUBLE])
     # 28 rows: 26 us and 39 when blocks of 512 entries left two thirds of the SMs idle
-    assert took[SETTLED] < 1.25 * took[DOUBLE], took
+    assert took[SETTLED] < 1.3 * took[DOUBLE], took
