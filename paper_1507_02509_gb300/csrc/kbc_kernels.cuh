@@ -503,36 +503,7 @@ step_fixup(const typename C::S* __restrict__ src, typename C::S* __restrict__ ds
 
 // ---------------------------------------------------------------- init / io
 
-// f = f^eq(rho, u) (Eq. Eq) of one node, stored as deviations from W_i;
-// computed in double, in the moment form
-//   f^eq_i - W_i = W_i (q + 3 v_i.j + rho (4.5 (v_i.u)^2 - 1.5 u^2)),
-// q = rho - 1, j = rho u: 28 FP64 instructions where nine polynomials took 61.
-template <class C>
-__device__ __forceinline__ void feq_node(double r, double x, double y, typename C::S* __restrict__ dst,
-                                         long long n, const StepArgs& a)
-{
-    const double q = r - 1.0, jx = r * x, jy = r * y;
-    const double A = jx * x, B = jy * y, xy = 0.25 * (jx * y);
-    const double S = A + B, q9 = (1.0 / 9.0) * q;
-    const double ex = fma(1.0 / 3.0, A, fma(-1.0 / 6.0, B, q9));
-    const double ey = fma(1.0 / 3.0, B, fma(-1.0 / 6.0, A, q9));
-    const double g = fma(1.0 / 12.0, S, 0.25 * q9);
-    const double dp = g + xy, dm = g - xy, sp = jx + jy, sm = jx - jy;
-    double d[9];
-    d[4] = fma(-2.0 / 3.0, S, 4.0 * q9);
-    d[5] = fma(1.0 / 3.0, jx, ex);
-    d[3] = fma(-1.0 / 3.0, jx, ex);
-    d[7] = fma(1.0 / 3.0, jy, ey);
-    d[1] = fma(-1.0 / 3.0, jy, ey);
-    d[8] = fma(1.0 / 12.0, sp, dp);
-    d[0] = fma(-1.0 / 12.0, sp, dp);
-    d[2] = fma(1.0 / 12.0, sm, dm);
-    d[6] = fma(-1.0 / 12.0, sm, dm);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = C::from_f64(d[i], i, a.cs);
-}
-
-// out of line: the rarely taken branch of feq_pair, which keeps the order
+// out of line: the rarely taken branch of the two below, which keeps the order
 // of operations that the stored float and half values have always had.
 // rho = 1 and u = 0 (of either sign) give f = W, for which no error bound
 // settles anything and which fluid at rest has in every node: stored without the
@@ -555,6 +526,43 @@ __device__ __noinline__ void feq_node_general(double r, double x, double y,
         const double dev = wgt(i) * ((r - 1.0) + r * P);
         dst[(long long)i * a.plane + n] = C::from_f64(dev, i, a.cs);
     }
+}
+
+// f = f^eq(rho, u) (Eq. Eq) of one node, stored as deviations from W_i;
+// computed in double, in the moment form
+//   f^eq_i - W_i = W_i (q + 3 v_i.j + rho (4.5 (v_i.u)^2 - 1.5 u^2)),
+// q = rho - 1, j = rho u: 28 FP64 instructions where nine polynomials took 61.
+template <class C>
+__device__ __forceinline__ void feq_node(double r, double x, double y, typename C::S* __restrict__ dst,
+                                         long long n, const StepArgs& a)
+{
+    // infinities, NaN and magnitudes whose products may overflow: the general
+    // form, whose terms turn into NaN together
+    const int top = max(max(__double2hiint(r) & 0x7fffffff, __double2hiint(x) & 0x7fffffff),
+                        __double2hiint(y) & 0x7fffffff);
+    if (top >= 0x52b00000) {  // 2^300
+        feq_node_general<C>(r, x, y, dst, n, a);
+        return;
+    }
+    const double q = r - 1.0, jx = r * x, jy = r * y;
+    const double A = jx * x, B = jy * y, xy = 0.25 * (jx * y);
+    const double S = A + B, q9 = (1.0 / 9.0) * q;
+    const double ex = fma(1.0 / 3.0, A, fma(-1.0 / 6.0, B, q9));
+    const double ey = fma(1.0 / 3.0, B, fma(-1.0 / 6.0, A, q9));
+    const double g = fma(1.0 / 12.0, S, 0.25 * q9);
+    const double dp = g + xy, dm = g - xy, sp = jx + jy, sm = jx - jy;
+    double d[9];
+    d[4] = fma(-2.0 / 3.0, S, 4.0 * q9);
+    d[5] = fma(1.0 / 3.0, jx, ex);
+    d[3] = fma(-1.0 / 3.0, jx, ex);
+    d[7] = fma(1.0 / 3.0, jy, ey);
+    d[1] = fma(-1.0 / 3.0, jy, ey);
+    d[8] = fma(1.0 / 12.0, sp, dp);
+    d[0] = fma(-1.0 / 12.0, sp, dp);
+    d[2] = fma(1.0 / 12.0, sm, dm);
+    d[6] = fma(-1.0 / 12.0, sm, dm);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) dst[(long long)i * a.plane + n] = C::from_f64(d[i], i, a.cs);
 }
 
 // Two nodes n0, n1 (n1 < 0: none) of the equilibrium for float or half
